@@ -1,0 +1,10 @@
+// kernels_line_yxf.cu -- y/x pass of the line path, size class 72 to 144, n1 = 72, 80, 90 (kernels_line.h).
+#include "kernels_line.cuh"
+
+namespace vloc {
+namespace line {
+template struct LaunchYX<2, 72>;
+template struct LaunchYX<2, 80>;
+template struct LaunchYX<2, 90>;
+}  // namespace line
+}  // namespace vloc

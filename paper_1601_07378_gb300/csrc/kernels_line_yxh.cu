@@ -1,0 +1,8 @@
+// kernels_line_yxh.cu -- y/x pass of the line path, size class 72 to 144, n1 = 100 (kernels_line.h).
+#include "kernels_line.cuh"
+
+namespace vloc {
+namespace line {
+template struct LaunchYX<2, 100>;
+}  // namespace line
+}  // namespace vloc

@@ -1,0 +1,8 @@
+// kernels_line_yxj.cu -- y/x pass of the line path, size class 72 to 144, n1 = 120 (kernels_line.h).
+#include "kernels_line.cuh"
+
+namespace vloc {
+namespace line {
+template struct LaunchYX<2, 120>;
+}  // namespace line
+}  // namespace vloc

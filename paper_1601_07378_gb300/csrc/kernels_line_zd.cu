@@ -1,0 +1,10 @@
+// kernels_line_zd.cu -- z-passes of the line path, lengths VLOC_LINE_Z_D (kernels_line.h).
+#include "kernels_line_z.cuh"
+
+namespace vloc {
+namespace line {
+#define VLOC_CASE(N) template struct LaunchZ<N>;
+VLOC_LINE_Z_D(VLOC_CASE)
+#undef VLOC_CASE
+}  // namespace line
+}  // namespace vloc

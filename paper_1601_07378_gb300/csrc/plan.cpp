@@ -23,6 +23,7 @@
 
 #include "../../include/vloc.h"
 #include "internal.h"
+#include "kernels_line.h"
 
 using namespace vloc;
 
@@ -132,6 +133,142 @@ FaultSpec fault_spec() {
     return f;
 }
 
+// Host tables of the line path; cls < 0: not for this plan (a length without
+// line kernels, or sticks outside the quarter band or with gaps along k in a
+// plane).
+struct LineHost {
+    int cls = -1, G = 0, runs = 0, trim = 0;
+    size_t o_gpos = 0, o_zd = 0, o_run = 0, o_ghp = 0, o_gh = 0, o_kr = 0;
+    std::vector<int> blob;
+};
+LineHost build_line(int n1, int n2, int n3, const std::vector<int>& stick_x, const std::vector<int>& stick_row,
+                    const std::vector<int>& pw_ptr, const std::vector<int>& pw_user, const std::vector<int>& pw_z,
+                    const std::vector<int32_t>& gamma_neg, int64_t nhalf) {
+    LineHost L;
+    const int cls = line::yx_class(n1, n2);
+    if (cls < 0 || !line::z_length(n3)) return L;
+    const int Q1 = n1 / 4, Q2 = n2 / 4, Q3 = n3 / 4, PP = line::class_pitch(cls);
+    const int S = (int)stick_x.size(), NPl = 2 * Q1 + 1;
+    std::vector<int> pos(S), kr(2 * NPl);
+    std::vector<int> count(NPl, 0);
+    for (int p = 0; p < NPl; ++p) { kr[2 * p] = 0; kr[2 * p + 1] = -1; }
+    for (int s = 0; s < S; ++s) {
+        const int h = stick_x[s] > n1 / 2 ? stick_x[s] - n1 : stick_x[s];
+        const int k = stick_row[s] > n2 / 2 ? stick_row[s] - n2 : stick_row[s];
+        if (h < -Q1 || h > Q1 || k < -Q2 || k > Q2) return L;
+        pos[s] = (k + Q2) * PP + h + Q1;
+        int* r = &kr[2 * (h + Q1)];
+        r[0] = std::min(r[0], k);
+        r[1] = std::max(r[1], k);
+        ++count[h + Q1];
+    }
+    for (int p = 0; p < NPl; ++p) {  // every k of the range present (k = 0 always within it)
+        if (count[p] != kr[2 * p + 1] - kr[2 * p] + 1) return L;
+        if (count[p] == 0) kr[2 * p] = 1;
+    }
+    // thin planes (at most two sticks) on both rims: as many as save the two
+    // warp pairs a round of 32-line groups, if any do
+    if (line::yx_thins(n1, n2)) {
+        auto rounds = [&](int w) { return line::yx_rounds(line::yx_bands(n1, n2) * (NPl - 2 * w)); };
+        for (int w = 1; w < Q1 && count[w - 1] <= 2 && count[NPl - w] <= 2; ++w)
+            if (rounds(w) < rounds(L.trim)) L.trim = w;
+    }
+    std::vector<int> order(S);
+    std::iota(order.begin(), order.end(), 0);
+    std::sort(order.begin(), order.end(), [&](int a, int b) { return pos[a] < pos[b]; });
+    // groups of 32 lanes (stick or -1)
+    std::vector<int> lanes;
+    const bool gamma = !gamma_neg.empty();
+    if (!gamma) {
+        for (int i = 0; i < S;) {  // aligned pairs of positions
+            const int a = order[i], b = i + 1 < S ? order[i + 1] : -1;
+            if (pos[a] & 1) { lanes.insert(lanes.end(), {-1, a}); ++i; }
+            else if (b >= 0 && pos[b] == pos[a] + 1) { lanes.insert(lanes.end(), {a, b}); i += 2; }
+            else { lanes.insert(lanes.end(), {a, -1}); ++i; }
+        }
+    } else {
+        // the list is symmetric, so the i-th stick from the front and from
+        // the back mirror each other (the middle one, if any, itself)
+        for (int i0 = 0; 2 * i0 < S; i0 += 16) {
+            const int m = std::min(16, (S + 1) / 2 - i0);
+            for (int j = 0; j < 16; ++j) lanes.push_back(j < m ? order[i0 + j] : -1);
+            for (int j = 15; j >= 0; --j) {
+                const bool self = j < m && 2 * (i0 + j) == S - 1;
+                lanes.push_back(j < m && !self ? order[S - 1 - i0 - j] : -1);
+            }
+        }
+    }
+    while (lanes.size() % 32) lanes.push_back(-1);
+    L.G = (int)(lanes.size() / 32);
+    std::vector<int> gpos(lanes.size());
+    for (size_t i = 0; i < lanes.size(); ++i) gpos[i] = lanes[i] < 0 ? -1 : pos[lanes[i]];
+    std::vector<int> zd, run, ghp, gh;
+    if (!gamma) {
+        // the rows of the first inverse stage that meet the band, as in the
+        // dense z-band table of the five-launch chain
+        int nst = 0, radix[4];
+        if (!plan_radices(n3, &nst, radix) || nst != 2) return L;
+        const int NA = n3 / radix[0];
+        std::vector<int> slot_of_row(n3, -1);
+        int rows = 0;
+        for (int r = 0; r < radix[0]; ++r) {
+            const int lo = r * NA, hi = lo + NA - 1;
+            if (lo <= Q3 || hi >= n3 - Q3) {
+                for (int i = 0; i < NA; ++i) slot_of_row[lo + i] = rows + i;
+                rows += NA;
+            }
+        }
+        zd.assign((size_t)L.G * rows * 32, -1);
+        run.assign((size_t)L.G * 32 * 4, 0);
+        L.runs = 1;  // every stick's plane waves consecutive in the caller's list, l ascending without a gap
+        for (size_t i = 0; i < lanes.size(); ++i) {
+            const int s = lanes[i];
+            if (s < 0) continue;
+            auto lsig = [&](int q) { return pw_z[q] > n3 / 2 ? pw_z[q] - n3 : pw_z[q]; };
+            const int q0 = pw_ptr[s], q1 = pw_ptr[s + 1];
+            for (int q = q0; q < q1; ++q) {
+                zd[((i / 32) * rows + slot_of_row[pw_z[q]]) * 32 + i % 32] = pw_user[q];
+                if (q > q0 && (pw_user[q] != pw_user[q - 1] + 1 || lsig(q) != lsig(q - 1) + 1)) L.runs = 0;
+            }
+            int* r = &run[4 * i];
+            r[0] = pw_user[q0]; r[1] = lsig(q0); r[2] = q1 - q0;
+        }
+    } else {
+        std::vector<int> group_of(pw_user.size(), -1), at_of(pw_user.size(), 0);
+        for (size_t i = 0; i < lanes.size(); ++i)
+            for (int s = lanes[i], q = s < 0 ? 0 : pw_ptr[s]; s >= 0 && q < pw_ptr[s + 1]; ++q) {
+                group_of[pw_user[q]] = (int)(i / 32);
+                at_of[pw_user[q]] = pw_z[q] | (int)(i % 32) << 16;
+            }
+        ghp.assign(L.G + 1, 0);
+        for (int64_t q = 0; q < nhalf; ++q) {
+            if (group_of[q] < 0 || group_of[q] != group_of[gamma_neg[q]]) return L;
+            ++ghp[group_of[q] + 1];
+        }
+        for (int g = 0; g < L.G; ++g) ghp[g + 1] += ghp[g];
+        std::vector<int> next(ghp.begin(), ghp.end() - 1);
+        gh.resize(4 * (size_t)nhalf);
+        for (int64_t q = 0; q < nhalf; ++q) {
+            int* e = &gh[4 * (size_t)next[group_of[q]]++];
+            e[0] = (int)q; e[1] = at_of[q]; e[2] = at_of[gamma_neg[q]]; e[3] = 0;
+        }
+    }
+    auto append = [&](const std::vector<int>& v) {
+        while (L.blob.size() & 3) L.blob.push_back(0);  // int4 alignment
+        const size_t off = L.blob.size();
+        L.blob.insert(L.blob.end(), v.begin(), v.end());
+        return off;
+    };
+    L.o_gpos = append(gpos);
+    L.o_zd = append(zd);
+    L.o_run = append(run);
+    L.o_ghp = append(ghp);
+    L.o_gh = append(gh);
+    L.o_kr = append(kr);
+    L.cls = cls;
+    return L;
+}
+
 }  // namespace
 
 struct vloc_plan_s {
@@ -167,6 +304,12 @@ struct vloc_plan_s {
     void* d_slab = nullptr;
     double* d_acc = nullptr;
     size_t ws_bytes = 0;
+    // line path (kernels_line.h): its tables; the dense bands share d_slab,
+    // the transposed V the start of d_acc
+    bool line_on = false;
+    vloc::line::Tables lt{};
+    void* d_line = nullptr;
+    size_t slab_bytes = 0;
     // host-buffer path (allocated on first use)
     void* d_stage = nullptr;
     size_t stage_bytes = 0;
@@ -231,6 +374,7 @@ static void free_plan(vloc_plan p) {
     cudaFree(p->d_vdf);
     cudaFree(p->d_err);
     cudaFree(p->d_gamma_buf);
+    cudaFree(p->d_line);
     cudaFree(p->d_stage);
     for (cudaEvent_t e : p->prof_pool) cudaEventDestroy(e);
     for (auto& g : p->graphs)
@@ -617,6 +761,12 @@ int vloc_plan_create(vloc_plan* out, int n1, int n2, int n3, const int32_t* g, i
         *out = p;
         return VLOC_OK;
     }
+    // ---- tables of the line path (not among the host tables: the
+    // allocation-free entry runs the five-launch chain)
+    LineHost lh;
+    if (!dbl && p->fast && p->lay.zq && !(flags & (VLOC_X_TMA | VLOC_Z_WARP | VLOC_Z_BULK)) &&
+        std::getenv("VLOC_GAMMA_PACK") == nullptr)
+        lh = build_line(n1, n2, n3, stick_x, stick_row, stick_pw_ptr, pw_user, pw_z, gamma_neg, npw_user);
     // shared-memory budget of the largest kernel tile
     int dev = 0;
     cudaError_t e;
@@ -637,6 +787,21 @@ int vloc_plan_create(vloc_plan* out, int n1, int n2, int n3, const int32_t* g, i
         free_plan(p); return cuda_fail(e, "upload tables");
     }
     p->dt = device_tables(p->d_tables, p->lay, n1, n2, n3, npw);
+    if (lh.cls >= 0) {
+        if ((e = dmalloc(&p->d_line, lh.blob.size() * sizeof(int)))) { free_plan(p); return cuda_fail(e, "cudaMalloc(line tables)"); }
+        if ((e = cudaMemcpyAsync(p->d_line, lh.blob.data(), lh.blob.size() * sizeof(int), cudaMemcpyHostToDevice, st))) {
+            free_plan(p); return cuda_fail(e, "upload line tables");
+        }
+        const int* base = (const int*)p->d_line;
+        line::Tables& t = p->lt;
+        t.gpos = base + lh.o_gpos; t.zd = base + lh.o_zd; t.run_tab = (const int4*)(base + lh.o_run);
+        t.gh_ptr = base + lh.o_ghp; t.gh = (const int4*)(base + lh.o_gh);
+        t.krange = (const int2*)(base + lh.o_kr);
+        t.gamma = p->gamma; t.runs = lh.runs; t.trim = lh.trim;
+        t.G = lh.G; t.n1 = n1; t.n2 = n2; t.n3 = n3; t.cls = lh.cls; t.npw = npw_user;
+        t.row = (2 * (n2 / 4) + 1) * line::class_pitch(lh.cls);
+        p->line_on = true;
+    }
     // the pair-forming z-passes exist for the FP32 compile-time kernels;
     // VLOC_GAMMA_PACK (a test aid) keeps the separate pack / unpack passes
     p->gfused = p->gamma && p->lay.gok && !dbl && p->fast && has_ct(n3) && std::getenv("VLOC_GAMMA_PACK") == nullptr;
@@ -678,9 +843,12 @@ int vloc_plan_create(vloc_plan* out, int n1, int n2, int n3, const int32_t* g, i
     p->chunk = chunk;
     p->ws_bands = std::max<long long>(chunk, 2);
     p->ngroups = (int)((std::max<long long>(1, p->ws_bands / 2) + kGradBandsPerGroup - 1) / kGradBandsPerGroup);
-    p->ws_bytes = per_band * (size_t)p->ws_bands + (size_t)N * sizeof(double) * (1 + p->ngroups);
+    // the line path's dense bands take the slab's place
+    const size_t slab_band = std::max((size_t)NP * n2 * n3 * elem, p->line_on ? line::band_elems(p->lt) * elem : (size_t)0);
+    p->slab_bytes = slab_band * (size_t)p->ws_bands;
+    p->ws_bytes = (size_t)S * n3 * elem * p->ws_bands + p->slab_bytes + (size_t)N * sizeof(double) * (1 + p->ngroups);
     if ((e = dmalloc((void**)&p->d_cyl, (size_t)S * n3 * elem * p->ws_bands))) { free_plan(p); return cuda_fail(e, "cudaMalloc(cylinder)"); }
-    if ((e = dmalloc((void**)&p->d_slab, (size_t)NP * n2 * n3 * elem * p->ws_bands))) { free_plan(p); return cuda_fail(e, "cudaMalloc(slab)"); }
+    if ((e = dmalloc((void**)&p->d_slab, p->slab_bytes))) { free_plan(p); return cuda_fail(e, "cudaMalloc(slab)"); }
     if (p->gamma) {
         if ((e = dmalloc((void**)&p->d_gamma_neg, sizeof(int) * (size_t)npw_user))) { free_plan(p); return cuda_fail(e, "cudaMalloc(gamma map)"); }
         if ((e = cudaMemcpyAsync(p->d_gamma_neg, gamma_neg.data(), sizeof(int) * (size_t)npw_user, cudaMemcpyHostToDevice, st))) {
@@ -718,6 +886,7 @@ int vloc_plan_create(vloc_plan* out, int n1, int n2, int n3, const int32_t* g, i
     }
 
     // dL/dV accumulator [N] followed by the band groups' partial sums [ngroups][N]
+    // (the line path's transposed V, N floats, shares it)
     if ((e = dmalloc((void**)&p->d_acc, (size_t)N * sizeof(double) * (1 + p->ngroups)))) { free_plan(p); return cuda_fail(e, "cudaMalloc(acc)"); }
     if ((e = cudaStreamSynchronize(st))) { free_plan(p); return cuda_fail(e, "plan create sync"); }
     *out = p;
@@ -740,6 +909,7 @@ int vloc_plan_set_schedule(vloc_plan p, int axis, int nst, const int32_t* radix)
     p->df = false;
     p->k3tma_on = false;
     p->gfused = false;
+    p->line_on = false;
     for (auto& g : p->graphs)
         if (g.exec) cudaGraphExecDestroy(g.exec);
     p->graphs.clear();
@@ -806,7 +976,7 @@ static int launch(vloc_plan p, int kind, cudaStream_t st, F&& f) {
 static int poison(vloc_plan p, cudaStream_t st) {
     if (!p->poison) return VLOC_OK;
     const size_t cyl = (size_t)p->S * p->n3 * p->elem * p->ws_bands;
-    const size_t slab = (size_t)p->NP * p->n2 * p->n3 * p->elem * p->ws_bands;
+    const size_t slab = p->slab_bytes;
     cudaError_t e;
     if ((e = cudaMemsetAsync(p->d_cyl, 0xFF, cyl, st))) return cuda_fail(e, "poison cylinder");
     if ((e = cudaMemsetAsync(p->d_slab, 0xFF, slab, st))) return cuda_fail(e, "poison slab");
@@ -815,10 +985,39 @@ static int poison(vloc_plan p, cudaStream_t st) {
 
 extern "C" {
 
+// Whether a call whose first chunk holds cb bands goes through the line path,
+// by its dense z rows (n3 x bands): three blocks of the y/x pass an SM.
+// Measured against the five launches (us): 4 bands at 96^3 39.5 against 37.2,
+// 5 41.1 / 41.3, 7 43 / 49, 3 at 144^3 79 / 74, 4 85 / 87, 10 at 48^3 23.5 /
+// 28.2.  (Smaller grids would gain from 200 rows on, 5 bands at 48^3 22.8 /
+// 24.7; results then depend on the chunk size for more calls.)  An axis
+// without the five launches' compile-time kernels leaves them behind at any
+// count (6 bands at 36^3 37 against 22).
+static bool line_chunk(vloc_plan p, long long cb) {
+    if (!p->line_on) return false;
+    return cb * p->n3 >= 456 || !(has_ct(p->n1) && has_ct(p->n2) && has_ct(p->n3));
+}
+static int line_vt(vloc_plan p, const void* V, cudaStream_t st) {
+    return launch(p, KK_AUX, st, [&] { return line::launch_vt((const float*)V, (float*)p->d_acc, p->lt, st); });
+}
+// One chunk of cb bands (Gamma: pairs of nreal real bands): inverse z, y/x, forward z.
+static int line_run(vloc_plan p, const void* c, long long cb, long long nreal, void* out, cudaStream_t st,
+                    const void* diag) {
+    float2* D = (float2*)p->d_slab;
+    int rc;
+    if ((rc = launch(p, KK_SCATTER_Z, st, [&] { return line::launch_z_inv(p->lt, (const float2*)p->d_tw[2], (const float2*)c, cb, nreal, D, st); }))) return rc;
+    if ((rc = launch(p, KK_X_V, st, [&] { return line::launch_yx(p->lt, (const float2*)p->d_tw[1], (const float*)p->d_acc, cb, D, st); }))) return rc;
+    return launch(p, KK_Z_GATHER, st, [&] {
+        return line::launch_z_fwd(p->lt, (const float2*)p->d_tw[2], D, cb, nreal, (float2*)out, (const float*)diag, (const float2*)c, st);
+    });
+}
+
 // out = A c over workspace chunks: K1, K2(+), K3, K2(-), K4 per chunk.
 // With `diag` (device real [npw]) the gather adds diag * c: out = (diag + A) c.
+// `call_bands` (0: nb): the bands of the caller's whole call where this is a
+// piece of it (host-buffer staging), so that every piece takes the same path.
 static int apply_impl(vloc_plan p, const void* c, const void* V, int64_t nb, void* out, cudaStream_t st,
-                      const void* diag = nullptr) {
+                      const void* diag = nullptr, int64_t call_bands = 0) {
     const size_t bstride = (size_t)p->npw * p->elem;
     const int dbl = p->dbl;
     const DevTables& t = p->dt;
@@ -840,12 +1039,21 @@ static int apply_impl(vloc_plan p, const void* c, const void* V, int64_t nb, voi
         }
         return VLOC_OK;
     }
+    // the line path for all chunks of a call or none (a Gamma plan's packed
+    // pairs, which come here, are not the caller's bands)
+    const bool line = !p->gamma && line_chunk(p, std::min<long long>(p->chunk, call_bands ? call_bands : nb));
+    if (line)
+        if (int rc = line_vt(p, V, st)) return rc;
     for (int64_t b0 = 0; b0 < nb; b0 += p->chunk) {
         const long long cb = std::min<long long>(p->chunk, nb - b0);
         const void* cc = (const char*)c + b0 * bstride;
         void* oo = (char*)out + b0 * bstride;
         int rc;
         if ((rc = poison(p, st))) return rc;
+        if (line) {
+            if ((rc = line_run(p, cc, cb, 0, oo, st, diag))) return rc;
+            continue;
+        }
         if ((rc = launch(p, KK_SCATTER_Z, st, [&] { return launch_k1_scatter_zpass(dbl, p->fast, t, ax, p->d_tw[2], cc, cb, p->d_cyl, st); }))) return rc;
         if ((rc = launch(p, KK_Y_INV, st, [&] { return launch_k2_ypass(dbl, p->fast, +1, t, ax, p->d_tw[1], cb, p->d_cyl, p->d_slab, st); }))) return rc;
         if ((rc = launch(p, KK_X_V, st, [&] { return launch_k3_xpass_v(dbl, p->fast, t, ax, p->d_tw[0], V, cb, p->d_slab, st, p->k3tma_on ? &p->k3tma : nullptr); }))) return rc;
@@ -887,8 +1095,21 @@ static int gamma_apply_fused(vloc_plan p, const void* c, const void* V, int64_t 
 
 static int gamma_apply(vloc_plan p, const void* c, const void* V, int64_t nb, void* out, cudaStream_t st,
                        const void* diag) {
-    if (p->gfused) return gamma_apply_fused(p, c, V, nb, out, st, diag);
     const long long npairs = (nb + 1) / 2;
+    // the line path for all chunks of a call or none
+    if (line_chunk(p, std::min<long long>(p->chunk, npairs))) {
+        if (int rc = line_vt(p, V, st)) return rc;
+        const size_t ustride = (size_t)p->npw_user * p->elem;
+        for (long long p0 = 0; p0 < npairs; p0 += p->chunk) {
+            const long long cp = std::min<long long>(p->chunk, npairs - p0);
+            const long long b0 = 2 * p0, bn = std::min<long long>(nb - b0, 2 * cp);
+            int rc;
+            if ((rc = poison(p, st))) return rc;
+            if ((rc = line_run(p, (const char*)c + b0 * ustride, cp, bn, (char*)out + b0 * ustride, st, diag))) return rc;
+        }
+        return VLOC_OK;
+    }
+    if (p->gfused) return gamma_apply_fused(p, c, V, nb, out, st, diag);
     const size_t full = (size_t)p->npw * p->elem;
     char* C = (char*)p->d_gamma_buf;
     char* U = C + (size_t)p->chunk * full;
@@ -1349,7 +1570,7 @@ static int apply_host_impl(vloc_plan p, const void* ch, const void* Vh, int64_t 
         if ((e = cudaEventRecord(p->ev[s], p->copy_stream))) return cuda_fail(e, "record");
         if ((e = cudaStreamWaitEvent(st, p->ev[s], 0))) return cuda_fail(e, "wait");
         if (used && (e = cudaStreamWaitEvent(st, p->ev[2 * K + s], 0))) return cuda_fail(e, "wait");
-        int rc = apply_impl(p, slot_in[s], dV, cb, slot_out[s], st);
+        int rc = apply_impl(p, slot_in[s], dV, cb, slot_out[s], st, nullptr, nb);
         if (rc) return rc;
         if ((e = cudaEventRecord(p->ev[K + s], st))) return cuda_fail(e, "record");
         if ((e = cudaStreamWaitEvent(p->d2h_stream, p->ev[K + s], 0))) return cuda_fail(e, "wait");
