@@ -23,7 +23,8 @@ ROOT = os.path.dirname(HERE)
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 SOURCES = ["kernels_ct_a.cu", "kernels_ct_b.cu", "kernels_ct_c.cu", "kernels_df_a.cu", "kernels_df_b.cu",
            "kernels_df_c.cu", "kernels_line.cu", *(f"kernels_line_yx{u}.cu" for u in "kjihgfedcba"),
-           *(f"kernels_line_z{u}.cu" for u in "dcba"), "kernels_f32.cu", "kernels_f64.cu", "kernels.cu", "plan.cpp", "noalloc.cu", "peaks.cu"]
+           *(f"kernels_line_z{u}.cu" for u in "dcba"), *(f"kernels_line_d{u}.cu" for u in "dcba"),
+            "kernels_f32.cu", "kernels_f64.cu", "kernels.cu", "plan.cpp", "noalloc.cu", "peaks.cu"]
 
 
 def _cuda_home() -> str:

@@ -74,6 +74,57 @@ int launch_z_fwd(const Tables& t, const float2* tw3, const float2* D, long long 
 }
 #undef VLOC_CASE_INV
 #undef VLOC_CASE_FWD
+int launch_dens(const Tables& t, const float2* D, long long nb, int bpg, const float* occ, long long b_base, int pair,
+                long long nreal, float* partial, cudaStream_t st) {
+#define VLOC_CASE0(N) case N: return LaunchDens<0, N>::run(t, D, nb, bpg, occ, b_base, pair, nreal, partial, st);
+#define VLOC_CASE1(N) case N: return LaunchDens<1, N>::run(t, D, nb, bpg, occ, b_base, pair, nreal, partial, st);
+#define VLOC_CASE2(N) case N: return LaunchDens<2, N>::run(t, D, nb, bpg, occ, b_base, pair, nreal, partial, st);
+    if (t.cls == 0) switch (t.n1) { VLOC_LINE_D48(VLOC_CASE0) default: break; }
+    if (t.cls == 1) switch (t.n1) { VLOC_LINE_D96(VLOC_CASE1) default: break; }
+    if (t.cls == 2) switch (t.n1) { VLOC_LINE_D144(VLOC_CASE2) default: break; }
+#undef VLOC_CASE0
+#undef VLOC_CASE1
+#undef VLOC_CASE2
+    return (int)cudaErrorInvalidValue;
+}
+// Tiles of 32 (y, z) at one x: the partial sums read along y, the result
+// written along z.  Sum over the groups as in k_reduce_partials_f32.
+__global__ void __launch_bounds__(256) k_dens_reduce(const float* __restrict__ partial, int ng, int n2, int n3,
+                                                     double* __restrict__ acc, int first, float* __restrict__ out) {
+    __shared__ float ts[32][33], tc[32][33];
+    const int z0 = blockIdx.x * 32, y0 = blockIdx.y * 32, x = blockIdx.z, n1 = gridDim.z;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const long long N = (long long)n1 * n2 * n3;
+    for (int j = ty; j < 32; j += 8) {
+        float s = 0.f, c = 0.f;
+        if (z0 + j < n3 && y0 + tx < n2) {
+            const float* q = partial + ((long long)(z0 + j) * n1 + x) * n2 + y0 + tx;
+#pragma unroll 4
+            for (int g = 0; g < ng; ++g) {
+                const float p = q[g * N];
+                const float t = __fadd_rn(s, p);
+                const float bp = __fsub_rn(t, s);  // the part of p that t took
+                c = __fadd_rn(c, __fadd_rn(__fsub_rn(s, __fsub_rn(t, bp)), __fsub_rn(p, bp)));
+                s = t;
+            }
+        }
+        ts[j][tx] = s;
+        tc[j][tx] = c;
+    }
+    __syncthreads();
+    for (int j = ty; j < 32; j += 8)
+        if (y0 + j < n2 && z0 + tx < n3) {
+            const long long i = ((long long)x * n2 + y0 + j) * n3 + z0 + tx;
+            const double tot = (first ? 0.0 : acc[i]) + ((double)ts[tx][j] + (double)tc[tx][j]);
+            if (out) out[i] = (float)tot;
+            else acc[i] = tot;
+        }
+}
+int launch_dens_reduce(const Tables& t, const float* partial, int ng, double* acc, int first, float* out,
+                       cudaStream_t st) {
+    k_dens_reduce<<<dim3((t.n3 + 31) / 32, (t.n2 + 31) / 32, t.n1), 256, 0, st>>>(partial, ng, t.n2, t.n3, acc, first, out);
+    return (int)cudaGetLastError();
+}
 int launch_yx(const Tables& t, const float2* tw2, const float* VT, long long nb, float2* D, cudaStream_t st) {
 #define VLOC_CASE0(N) case N: return LaunchYX<0, N>::run(t, tw2, VT, nb, D, st);
 #define VLOC_CASE1(N) case N: return LaunchYX<1, N>::run(t, tw2, VT, nb, D, st);

@@ -94,16 +94,16 @@ struct YXStep {
 // inverse one: the forward transform is the inverse of the conjugate, and the
 // conjugation rides on the multiply by V and on the final store.  (Two bodies
 // instead of four keep the code of a step small enough for the instruction
-// cache; with four the kernel was held up by instruction fetches.)  DX, DY:
-// whether kind 1 / kinds 0 and 2 are wanted of this length (both for n1 = n2).
-template <int N, class C, int N2, bool DX, bool DY>
+// cache; with four the kernel was held up by instruction fetches.)  KINDS: bit
+// set of the kinds wanted of this length (all three for n1 = n2).
+template <int N, class C, int N2, int KINDS>
 __device__ __forceinline__ void yx_body(int kind_, const YXStep& s) {
     constexpr int M = N / 2, Q = N / 4, AP = C::AP, PP = C::PP, SLOT = C::SLOT, PAIRS = C::PAIRS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float2* const A = reinterpret_cast<float2*>(smem_raw);
     const int lane = threadIdx.x & 31, role = (threadIdx.x >> 5) & 1, pair = threadIdx.x >> 6;
     asm volatile("" : "+r"(kind_));  // one body for the kinds, not a specialised copy of each
-    const int kind = !DX ? kind_ & 2 : !DY ? 1 : kind_;
+    const int kind = KINDS == 7 ? kind_ : KINDS == 5 ? kind_ & 2 : KINDS == 2 ? 1 : 0;
     const int per = kind == 1 ? N2 : s.planes, p0 = kind == 1 ? 0 : s.p0, lines = per * s.nbb;
 #pragma unroll 1
     for (int l0 = pair * 32; l0 < lines; l0 += PAIRS * 32) {
@@ -244,10 +244,10 @@ __global__ void __launch_bounds__(64 * YX<CLS, N1, N2>::PAIRS, YX<CLS, N1, N2>::
         for (int kind = 0; kind < 3; ++kind) {
             if (b > b0 || kind > 0) __syncthreads();  // the last phase's rows are written, or have been read
             if constexpr (N1 == N2) {
-                yx_body<N1, C, N2, true, true>(kind, s);
+                yx_body<N1, C, N2, 7>(kind, s);
             } else {
-                if (kind == 1) yx_body<N1, C, N2, true, false>(kind, s);
-                else yx_body<N2, C, N2, false, true>(kind, s);
+                if (kind == 1) yx_body<N1, C, N2, 2>(kind, s);
+                else yx_body<N2, C, N2, 5>(kind, s);
             }
             if constexpr (yx_thins(N1, N2))
                 if (kind != 1) yx_thin<C, N2>(kind == 2, s);

@@ -84,12 +84,29 @@ int launch_yx(const Tables& t, const float2* tw2, const float* VT, long long nb,
 int launch_z_fwd(const Tables& t, const float2* tw3, const float2* D, long long nb, long long nreal, float2* out,
                  const float* diag, const float2* c, cudaStream_t st);
 
+// Density: partial sums [group][z][x][y] of groups of at most bpg bands of D
+// (see launch_k3d_density), and their sum over the ng groups, in order and
+// compensated as launch_reduce_partials_f32, turned to [x][y][z]
+int launch_dens(const Tables& t, const float2* D, long long nb, int bpg, const float* occ, long long b_base, int pair,
+                long long nreal, float* partial, cudaStream_t st);
+int launch_dens_reduce(const Tables& t, const float* partial, int ng, double* acc, int first, float* out,
+                       cudaStream_t st);
+
 // instantiated per length / class in kernels_line_*.cu
 template <int N> struct LaunchZ {
     static int inv(const Tables& t, const float2* tw3, const float2* c, long long nb, long long nreal, float2* D,
                    cudaStream_t st);
     static int fwd(const Tables& t, const float2* tw3, const float2* D, long long nb, long long nreal, float2* out,
                    const float* diag, const float2* c, cudaStream_t st);
+};
+// the density of n1 with compile-time density kernels in the five-launch chain
+// (elsewhere the group sums are FP64)
+#define VLOC_LINE_D48(X) X(24) X(32) X(48)
+#define VLOC_LINE_D96(X) X(48) X(60) X(64) X(72) X(80) X(96)
+#define VLOC_LINE_D144(X) X(72) X(80) X(96) X(100) X(120) X(128) X(144)
+template <int CLS, int N1> struct LaunchDens {
+    static int run(const Tables& t, const float2* D, long long nb, int bpg, const float* occ, long long b_base, int pair,
+                   long long nreal, float* partial, cudaStream_t st);
 };
 template <int CLS, int N1> struct LaunchYX {
     static int run(const Tables& t, const float2* tw2, const float* VT, long long nb, float2* D, cudaStream_t st);

@@ -1369,6 +1369,38 @@ int vloc_density(vloc_plan p, const void* c, const void* occ, int64_t nb, void* 
     const bool fused = pf32 && nb > 0;
     bool first = true;
     if (!fused && (rc = launch(p, KK_AUX, st, [&] { return launch_zero_f64(p->d_acc, p->N, st); }))) return rc;
+    // The line path's z-pass and y/x density pass, for all chunks or none.
+    // Its blocks take a band at a time, so n2 <= 32 leaves one of the two warp
+    // pairs idle (32^3 x 300 bands 56 against 45 us); above, the two ways
+    // measured 536 and 616 us at 96^3 x 300, 840 / 1197 at 100^3, 1210 / 1875
+    // at 120^3, 1518 / 1526 at 128^3, 52.9 / 63.1 at 64^3 x 64.  Smaller groups
+    // where the grid of 16-band groups leaves SMs idle (each group costs a
+    // partial grid).
+    if (fused && p->n2 > 32 && line_chunk(p, std::min<long long>(p->chunk, p->gamma ? (nb + 1) / 2 : nb))) {
+        const long long pairs = p->gamma ? (nb + 1) / 2 : nb;  // complex bands
+        float2* Dl = (float2*)p->d_slab;
+        for (long long j0 = 0; j0 < pairs;) {
+            const long long cb = std::min(std::min<long long>(p->chunk, per_pass), pairs - j0);
+            int bpg = (int)kGradBandsPerGroup;
+            while (bpg > 2 && (cb + bpg / 2 - 1) / (bpg / 2) <= 2 * p->ngroups && p->n3 * ((cb + bpg - 1) / bpg) < 912) bpg /= 2;
+            const int ng = (int)((cb + bpg - 1) / bpg);
+            if ((rc = poison(p, st))) return rc;
+            const float2* src = (const float2*)c + (p->gamma ? 2 : 1) * j0 * p->npw_user;
+            if ((rc = launch(p, KK_SCATTER_Z, st, [&] {
+                     return line::launch_z_inv(p->lt, (const float2*)p->d_tw[2], src, cb, nb - 2 * j0, Dl, st);
+                 }))) return rc;
+            if ((rc = launch(p, KK_DENSITY, st, [&] {
+                     return line::launch_dens(p->lt, Dl, cb, bpg, (const float*)occ, j0, p->gamma, nb, (float*)partial, st);
+                 }))) return rc;
+            j0 += cb;
+            if ((rc = launch(p, KK_AUX, st, [&] {
+                     return line::launch_dens_reduce(p->lt, (const float*)partial, ng, p->d_acc, first,
+                                                     j0 >= pairs ? (float*)rho : nullptr, st);
+                 }))) return rc;
+            first = false;
+        }
+        return VLOC_OK;
+    }
     // K1 + K2 on `cb` complex bands at `src` (stride npw), then the density
     // x-pass; `base` is the global index of the chunk's first (pair) band,
     // `last` says that no chunk follows.

@@ -124,3 +124,35 @@ def test_line_path_lists_chunks_and_misaligned_buffers(monkeypatch):
     p2 = vloc.VlocPlan(n, g2, torch.complex64)
     assert _launches(p2, lambda: p2.apply(torch.zeros((40, len(g2)), dtype=torch.complex64, device="cuda"), Vt))[1] == 5
     assert _launches(p, lambda: p.apply(ct[:6], Vt))[1] == 5
+
+
+# lengths with compile-time density kernels on x (the others keep their FP64
+# group sums); group sizes 2, 4, 8 and 16, ragged last groups, several chunks
+@pytest.mark.parametrize("n,R,nb,chunk,gamma", [((32, 36, 24), 6.0, 23, 0, False), ((48, 40, 36), 9.0, 37, 14, False),
+                                                ((64, 64, 64), 16.0, 67, 0, False), ((96, 72, 30), 7.5, 131, 0, False),
+                                                ((100, 108, 24), 6.0, 90, 40, False), ((128, 128, 32), 8.0, 33, 0, False),
+                                                ((144, 120, 24), 6.0, 20, 0, False), ((60, 64, 48), 12.0, 45, 0, True),
+                                                ((96, 96, 24), 6.0, 87, 20, True)])
+def test_line_density(n, R, nb, chunk, gamma, monkeypatch):
+    g = synth.sphere_glist(*n, R, order="shuffled", seed=6)
+    if gamma:
+        g = synth.half_sphere(g)
+    c = synth.coefficients(g, nb, seed=206).astype(np.complex64)
+    if gamma:
+        zero = np.flatnonzero(~g.any(axis=1))
+        c[:, zero] = c[:, zero].real
+    occ = np.linspace(2.0, 0.25, nb).astype(np.float32)
+    p, ref = _plans(n, g, monkeypatch, chunk=chunk, gamma=gamma, poison=True)
+    ct, ot = torch.from_numpy(c).cuda(), torch.from_numpy(occ).cuda()
+    rho, launches = _launches(p, lambda: p.density(ct, ot))
+    m = (nb + 1) // 2 if gamma else nb
+    assert launches == 3 * (-(-m // chunk) if chunk else 1)    # the line path: three launches a chunk
+    rho0 = ref.density(ct, ot)
+    ones = p.density(ct)
+    assert torch.equal(rho, p.density(ct, ot))
+    f = O.gamma_density if gamma else O.density
+    want = f(n, g, c.astype(np.complex128), occ.astype(np.float64))
+    err = lambda a, b: np.linalg.norm(a.cpu().numpy().astype(np.float64) - b) / np.linalg.norm(b)
+    assert err(rho, want) < TOL["f32"]
+    assert err(rho, rho0.cpu().numpy().astype(np.float64)) < 3e-7
+    assert err(ones, f(n, g, c.astype(np.complex128), np.ones(nb))) < TOL["f32"]
