@@ -9,6 +9,7 @@
 
 #include "internal.h"
 #include "fft_core.cuh"
+#include "pdl.cuh"
 
 namespace vloc {
 
@@ -121,12 +122,12 @@ int launch_twiddles_df(const void* tw64, void* twdf, int n, cudaStream_t st) {
     return (int)cudaGetLastError();
 }
 __global__ void k_v_to_df(const double* __restrict__ V, float2* __restrict__ out, long long N) {
+    pdl_begin();
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (i < N) out[i] = df_split(V[i]);
 }
 int launch_v_to_df(const void* V, void* Vdf, long long N, cudaStream_t st) {
-    k_v_to_df<<<(unsigned)((N + 255) / 256), 256, 0, st>>>((const double*)V, (float2*)Vdf, N);
-    return (int)cudaGetLastError();
+    return pdl_launch(k_v_to_df, (unsigned)((N + 255) / 256), 256, 0, st, (const double*)V, (float2*)Vdf, N);
 }
 
 bool has_ct(int n) {

@@ -354,6 +354,7 @@ template <int N, bool GM = false>
 __global__ void __launch_bounds__(kThreads, minb_k1(N)) k1_ct(DevTables t, const float2* __restrict__ tw3,
                                                  const float2* __restrict__ coeffs, float2* __restrict__ cyl,
                                                  GammaArgs g) {
+    pdl_begin();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float2* buf = reinterpret_cast<float2*>(smem_raw);
     float2* stw = buf + N * kLdP;
@@ -380,6 +381,7 @@ template <int N, bool GM = false>
 __global__ void __launch_bounds__(kThreads, minb_k1(N)) k1q_ct(DevTables t, const float2* __restrict__ tw3,
                                                   const float2* __restrict__ coeffs, float2* __restrict__ cyl,
                                                   GammaArgs g) {
+    pdl_begin();
     using SC = Sched<N>;
     static_assert(SC::nst == 2, "quarter-band z-pass: two-stage lengths");
     using QR = QRows<N>;
@@ -482,6 +484,7 @@ __global__ void __launch_bounds__(kThreads, minb_k1(N)) k1q_ct(DevTables t, cons
 template <int N, bool RUNS>
 __global__ void __launch_bounds__(kThreads, minb_k1(N)) k1d_ct(DevTables t, const float2* __restrict__ tw3,
                                                   const float2* __restrict__ coeffs, float2* __restrict__ cyl) {
+    pdl_begin();
     using SC = Sched<N>;
     static_assert(SC::nst == 2, "quarter-band z-pass: two-stage lengths");
     using QR = QRows<N>;
@@ -662,6 +665,7 @@ __global__ void __launch_bounds__(kThreads, minb_k1(N)) k1b_ct(DevTables t, cons
 template <int S, int N>
 __global__ void __launch_bounds__(kThreads, minb_k2(N, S)) k2_ct(DevTables t, const float2* __restrict__ tw2, float2* cyl,
                                                  float2* slab) {
+    pdl_begin();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int n3 = t.n3;
     float2* buf = reinterpret_cast<float2*>(smem_raw);
@@ -688,6 +692,7 @@ __global__ void __launch_bounds__(kThreads, minb_k2(N, S)) k2_ct(DevTables t, co
 template <int N, int W>
 __global__ void __launch_bounds__(32 * W, minb_k3(N)) k3_ct(DevTables t, const float2* __restrict__ tw1,
                                                  const float* __restrict__ Vr, float2* slab) {
+    pdl_begin();
     using SC = Sched<N>;
     constexpr int nst = SC::nst;
     static_assert(nst >= 2, "compile-time x-pass needs at least two stages");
@@ -805,6 +810,7 @@ constexpr int minb_k3q(int n) {
 template <int N, int W, bool FLAT = true>
 __global__ void __launch_bounds__(32 * W, minb_k3q(N)) k3q_ct(DevTables t, const float2* __restrict__ tw1,
                                                   const float* __restrict__ Vr, float2* slab) {
+    pdl_begin();
     using SC = Sched<N>;
     static_assert(SC::nst == 2, "quarter-sphere x-pass: two-stage lengths");
     using QR = QRows<N>;
@@ -973,6 +979,7 @@ template <int N, bool GM = false>
 __global__ void __launch_bounds__(kThreads, minb_k4(N)) k4_ct(DevTables t, const float2* __restrict__ tw3,
                                                  const float2* __restrict__ cyl, float2* out, float scale,
                                                  const float* __restrict__ diag, const float2* cin, GammaArgs g) {
+    pdl_begin();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float2* buf = reinterpret_cast<float2*>(smem_raw);
     float2* stw = buf + N * kLdP;
@@ -999,6 +1006,7 @@ template <int N, bool GM = false>
 __global__ void __launch_bounds__(kThreads, minb_k4q(N, GM)) k4q_ct(DevTables t, const float2* __restrict__ tw3,
                                                   const float2* __restrict__ cyl, float2* out, float scale,
                                                   const float* __restrict__ diag, const float2* cin, GammaArgs g) {
+    pdl_begin();
     using SC = Sched<N>;
     static_assert(SC::nst == 2, "quarter-band z-pass: two-stage lengths");
     using QR = QRows<N>;
@@ -1055,6 +1063,7 @@ template <int N>
 __global__ void __launch_bounds__(kThreads, minb_k4d(N)) k4d_ct(DevTables t, const float2* __restrict__ tw3,
                                                   const float2* __restrict__ cyl, float2* out, float scale,
                                                   const float* __restrict__ diag, const float2* cin) {
+    pdl_begin();
     using SC = Sched<N>;
     static_assert(SC::nst == 2, "quarter-band z-pass: two-stage lengths");
     using QR = QRows<N>;
@@ -1546,30 +1555,25 @@ int launch_k1_ct(const DevTables& t, const void* tw3, const void* coeffs, long l
             if (t.runs == 2) {
                 static const cudaError_t oncer = CtSmem<N>::ensure(k1d_ct<N, true>);
                 if (oncer) return (int)oncer;
-                k1d_ct<N, true><<<dim3(t.T, (unsigned)nb), kThreads, CtSmem<N>::sm, st>>>(t, (const float2*)tw3,
-                                                                                      (const float2*)coeffs, (float2*)cyl);
-                return (int)cudaGetLastError();
+                return pdl_launch(k1d_ct<N, true>, dim3(t.T, (unsigned)nb), kThreads, CtSmem<N>::sm, st, t, (const
+                    float2*)tw3, (const float2*)coeffs, (float2*)cyl);
             }
             static const cudaError_t onced = CtSmem<N>::ensure(k1d_ct<N, false>);
             if (onced) return (int)onced;
-            k1d_ct<N, false><<<dim3(t.T, (unsigned)nb), kThreads, CtSmem<N>::sm, st>>>(t, (const float2*)tw3,
-                                                                                       (const float2*)coeffs, (float2*)cyl);
-            return (int)cudaGetLastError();
+            return pdl_launch(k1d_ct<N, false>, dim3(t.T, (unsigned)nb), kThreads, CtSmem<N>::sm, st, t, (const
+                float2*)tw3, (const float2*)coeffs, (float2*)cyl);
         }
         if (t.zq) {
             static const cudaError_t onceq = CtSmem<N>::ensure(k1q_ct<N, GM>);
             if (onceq) return (int)onceq;
-            k1q_ct<N, GM><<<dim3(t.T, (unsigned)nb), kThreads, CtSmem<N>::sm, st>>>(t, (const float2*)tw3,
-                                                                                    (const float2*)coeffs,
-                                                                                    (float2*)cyl, g);
-            return (int)cudaGetLastError();
+            return pdl_launch(k1q_ct<N, GM>, dim3(t.T, (unsigned)nb), kThreads, CtSmem<N>::sm, st, t, (const
+                float2*)tw3, (const float2*)coeffs, (float2*)cyl, g);
         }
     }
     static const cudaError_t once = CtSmem<N>::ensure(k1_ct<N, GM>);
     if (once) return (int)once;
-    k1_ct<N, GM><<<dim3(t.T, (unsigned)nb), kThreads, CtSmem<N>::sm, st>>>(t, (const float2*)tw3,
-                                                                           (const float2*)coeffs, (float2*)cyl, g);
-    return (int)cudaGetLastError();
+    return pdl_launch(k1_ct<N, GM>, dim3(t.T, (unsigned)nb), kThreads, CtSmem<N>::sm, st, t, (const float2*)tw3,
+        (const float2*)coeffs, (float2*)cyl, g);
 }
 template <typename T, int N>
 int LaunchCT<T, N>::k1(const DevTables& t, const void* tw3, const void* coeffs, long long nb, void* cyl,
@@ -1589,13 +1593,14 @@ int LaunchCT<T, N>::k2(int sign, const DevTables& t, const void* tw2, long long 
     if (sign > 0) {
         static const cudaError_t once = CtSmem<N>::ensure(k2_ct<+1, N>);
         if (once) return (int)once;
-        k2_ct<+1, N><<<grid, kThreads, CtSmem<N>::sm, st>>>(t, (const float2*)tw2, (float2*)cyl, (float2*)slab);
+        return pdl_launch(k2_ct<+1, N>, grid, kThreads, CtSmem<N>::sm, st, t, (const float2*)tw2, (float2*)cyl,
+            (float2*)slab);
     } else {
         static const cudaError_t once = CtSmem<N>::ensure(k2_ct<-1, N>);
         if (once) return (int)once;
-        k2_ct<-1, N><<<grid, kThreads, CtSmem<N>::sm, st>>>(t, (const float2*)tw2, (float2*)cyl, (float2*)slab);
+        return pdl_launch(k2_ct<-1, N>, grid, kThreads, CtSmem<N>::sm, st, t, (const float2*)tw2, (float2*)cyl,
+            (float2*)slab);
     }
-    return (int)cudaGetLastError();
 }
 // defined in k3_tma.cuh (included by the instantiating files)
 template <int N> int launch_k3_tma(const DevTables& t, const void* tw1, const void* V, long long nb, void* slab,
@@ -1613,20 +1618,20 @@ int LaunchCT<T, N>::k3(const DevTables& t, const void* tw1, const void* V, long 
             static_assert(sm <= 48 * 1024, "x-pass tile within the default shared-memory limit");
             if (t.n3 % kLines == 0) {
                 const dim3 grid(t.n2, t.n3 / kLines, (unsigned)nb);
-                k3q_ct<N, W, false><<<grid, 32 * W, sm, st>>>(t, (const float2*)tw1, (const float*)V, (float2*)slab);
+                return pdl_launch(k3q_ct<N, W, false>, grid, 32 * W, sm, st, t, (const float2*)tw1, (const float*)V,
+                    (float2*)slab);
             } else {
                 const dim3 grid((unsigned)((t.n2 * (t.n3 / 2) + 15) / 16), 1, (unsigned)nb);  // 16 line pairs a tile
-                k3q_ct<N, W, true><<<grid, 32 * W, sm, st>>>(t, (const float2*)tw1, (const float*)V, (float2*)slab);
+                return pdl_launch(k3q_ct<N, W, true>, grid, 32 * W, sm, st, t, (const float2*)tw1, (const float*)V,
+                    (float2*)slab);
             }
-            return (int)cudaGetLastError();
         }
     }
     static const cudaError_t once = CtSmem<N>::ensure(k3_ct<N, W>);
     if (once) return (int)once;
     const dim3 grid(t.n2, (t.n3 + kLines - 1) / kLines, (unsigned)nb);
-    k3_ct<N, W><<<grid, 32 * W, CtSmem<N>::sm, st>>>(t, (const float2*)tw1, (const float*)V,
-                                                                           (float2*)slab);
-    return (int)cudaGetLastError();
+    return pdl_launch(k3_ct<N, W>, grid, 32 * W, CtSmem<N>::sm, st, t, (const float2*)tw1, (const float*)V,
+        (float2*)slab);
 }
 template <typename T, int N>
 int LaunchCT<T, N>::k3b(const DevTables& t, const void* tw1, const void* sc, const void* sg, long long nb, int bpg,
@@ -1703,24 +1708,20 @@ int launch_k4_ct(const DevTables& t, const void* tw3, const void* cyl, long long
         if (!GM && VLOC_K4_DIRECT && t.zd_rows == QRows<N>::groups() * QRows<N>::NA) {
             static const cudaError_t onced = CtSmem<N>::ensure(k4d_ct<N>);
             if (onced) return (int)onced;
-            k4d_ct<N><<<dim3(t.T, (unsigned)nb), kThreads, CtSmem<N>::sm, st>>>(
-                t, (const float2*)tw3, (const float2*)cyl, (float2*)out, scale, (const float*)diag, (const float2*)cin);
-            return (int)cudaGetLastError();
+            return pdl_launch(k4d_ct<N>, dim3(t.T, (unsigned)nb), kThreads, CtSmem<N>::sm, st, t, (const float2*)tw3,
+                (const float2*)cyl, (float2*)out, scale, (const float*)diag, (const float2*)cin);
         }
         if (t.zq) {
             static const cudaError_t onceq = CtSmem<N>::ensure(k4q_ct<N, GM>);
             if (onceq) return (int)onceq;
-            k4q_ct<N, GM><<<dim3(t.T, (unsigned)nb), kThreads, CtSmem<N>::sm, st>>>(
-                t, (const float2*)tw3, (const float2*)cyl, (float2*)out, scale, (const float*)diag, (const float2*)cin,
-                g);
-            return (int)cudaGetLastError();
+            return pdl_launch(k4q_ct<N, GM>, dim3(t.T, (unsigned)nb), kThreads, CtSmem<N>::sm, st, t, (const
+                float2*)tw3, (const float2*)cyl, (float2*)out, scale, (const float*)diag, (const float2*)cin, g);
         }
     }
     static const cudaError_t once = CtSmem<N>::ensure(k4_ct<N, GM>);
     if (once) return (int)once;
-    k4_ct<N, GM><<<dim3(t.T, (unsigned)nb), kThreads, CtSmem<N>::sm, st>>>(
-        t, (const float2*)tw3, (const float2*)cyl, (float2*)out, scale, (const float*)diag, (const float2*)cin, g);
-    return (int)cudaGetLastError();
+    return pdl_launch(k4_ct<N, GM>, dim3(t.T, (unsigned)nb), kThreads, CtSmem<N>::sm, st, t, (const float2*)tw3,
+        (const float2*)cyl, (float2*)out, scale, (const float*)diag, (const float2*)cin, g);
 }
 template <typename T, int N>
 int LaunchCT<T, N>::k4(const DevTables& t, const void* tw3, const void* cyl, long long nb, void* out,

@@ -170,12 +170,14 @@ template <class Pol, int N> constexpr bool df_floors() { return std::is_same<Pol
 template <class Pol, int N>
 __global__ void __launch_bounds__(kThreads) k1_w(DevTables t, const typename Pol::TW* __restrict__ tw3,
                                                 const double2* __restrict__ coeffs, typename Pol::V* __restrict__ cyl) {
+    pdl_begin();
     k1w_body<Pol, N>(t, tw3, coeffs, cyl);
 }
 template <class Pol, int N, int MINB>
 __global__ void __launch_bounds__(kThreads, MINB) k1_wb(DevTables t, const typename Pol::TW* __restrict__ tw3,
                                                        const double2* __restrict__ coeffs,
                                                        typename Pol::V* __restrict__ cyl) {
+    pdl_begin();
     k1w_body<Pol, N>(t, tw3, coeffs, cyl);
 }
 
@@ -249,12 +251,14 @@ __device__ __forceinline__ void k1dw_body(const DevTables& t, const typename Pol
 template <class Pol, int N>
 __global__ void __launch_bounds__(kThreads) k1d_w(DevTables t, const typename Pol::TW* __restrict__ tw3,
                                                  const double2* __restrict__ coeffs, typename Pol::V* __restrict__ cyl) {
+    pdl_begin();
     k1dw_body<Pol, N>(t, tw3, coeffs, cyl);
 }
 template <class Pol, int N, int MINB>
 __global__ void __launch_bounds__(kThreads, MINB) k1d_wb(DevTables t, const typename Pol::TW* __restrict__ tw3,
                                                         const double2* __restrict__ coeffs,
                                                         typename Pol::V* __restrict__ cyl) {
+    pdl_begin();
     k1dw_body<Pol, N>(t, tw3, coeffs, cyl);
 }
 
@@ -291,11 +295,13 @@ __device__ __forceinline__ void k2w_body(const DevTables& t, const typename Pol:
 template <class Pol, int S, int N>
 __global__ void __launch_bounds__(kThreads) k2_w(DevTables t, const typename Pol::TW* __restrict__ tw2,
                                                 typename Pol::V* cyl, typename Pol::V* slab) {
+    pdl_begin();
     k2w_body<Pol, S, N>(t, tw2, cyl, slab);
 }
 template <class Pol, int S, int N, int MINB>
 __global__ void __launch_bounds__(kThreads, MINB) k2_wb(DevTables t, const typename Pol::TW* __restrict__ tw2,
                                                        typename Pol::V* cyl, typename Pol::V* slab) {
+    pdl_begin();
     k2w_body<Pol, S, N>(t, tw2, cyl, slab);
 }
 
@@ -305,6 +311,7 @@ __global__ void __launch_bounds__(kThreads, MINB) k2_wb(DevTables t, const typen
 template <class Pol, int N>
 __global__ void __launch_bounds__(kThreads) k3_w(DevTables t, const typename Pol::TW* __restrict__ tw1,
                                                 const typename Pol::VR* __restrict__ Vr, typename Pol::V* slab) {
+    pdl_begin();
     using V = typename Pol::V;
     using TW = typename Pol::TW;
     using SC = Sched<N>;
@@ -383,6 +390,7 @@ template <class Pol, int N> __host__ __device__ constexpr size_t k3q_w_smem() {
 template <class Pol, int N>
 __global__ void __launch_bounds__(kThreads) k3q_w(DevTables t, const typename Pol::TW* __restrict__ tw1,
                                                  const typename Pol::VR* __restrict__ Vr, typename Pol::V* slab) {
+    pdl_begin();
     using V = typename Pol::V;
     using TW = typename Pol::TW;
     using SC = Sched<N>;
@@ -531,6 +539,7 @@ template <class Pol, int N>
 __global__ void __launch_bounds__(kThreads) k4_w(DevTables t, const typename Pol::TW* __restrict__ tw3,
                                                 const typename Pol::V* __restrict__ cyl, double2* out, double scale,
                                                 const double* __restrict__ diag, const double2* cin) {
+    pdl_begin();
     k4w_body<Pol, N>(t, tw3, cyl, out, scale, diag, cin);
 }
 template <class Pol, int N, int MINB>
@@ -538,6 +547,7 @@ __global__ void __launch_bounds__(kThreads, MINB) k4_wb(DevTables t, const typen
                                                        const typename Pol::V* __restrict__ cyl, double2* out,
                                                        double scale, const double* __restrict__ diag,
                                                        const double2* cin) {
+    pdl_begin();
     k4w_body<Pol, N>(t, tw3, cyl, out, scale, diag, cin);
 }
 
@@ -559,29 +569,27 @@ int LaunchF64<P, N>::k1(const DevTables& t, const void* tw3, const void* coeffs,
             if constexpr (df_floors<Pol, N>()) {
                 static const cudaError_t onced = WSmem<Pol, N>::ensure(k1d_wb<Pol, N, VLOC_MINB_K1DF>);
                 if (onced) return (int)onced;
-                k1d_wb<Pol, N, VLOC_MINB_K1DF><<<dim3(t.T, (unsigned)nb, 2), kThreads, WSmem<Pol, N>::sm, st>>>(
-                    t, (const typename Pol::TW*)tw3, (const double2*)coeffs, (typename Pol::V*)cyl);
+                return pdl_launch(k1d_wb<Pol, N, VLOC_MINB_K1DF>, dim3(t.T, (unsigned)nb, 2), kThreads, WSmem<Pol,
+                    N>::sm, st, t, (const typename Pol::TW*)tw3, (const double2*)coeffs, (typename Pol::V*)cyl);
             } else {
                 static const cudaError_t onced = WSmem<Pol, N>::ensure(k1d_w<Pol, N>);
                 if (onced) return (int)onced;
-                k1d_w<Pol, N><<<dim3(t.T, (unsigned)nb, 2), kThreads, WSmem<Pol, N>::sm, st>>>(
-                    t, (const typename Pol::TW*)tw3, (const double2*)coeffs, (typename Pol::V*)cyl);
+                return pdl_launch(k1d_w<Pol, N>, dim3(t.T, (unsigned)nb, 2), kThreads, WSmem<Pol, N>::sm, st, t,
+                    (const typename Pol::TW*)tw3, (const double2*)coeffs, (typename Pol::V*)cyl);
             }
-            return (int)cudaGetLastError();
         }
     }
     if constexpr (df_floors<Pol, N>()) {
         static const cudaError_t onceb = WSmem<Pol, N>::ensure(k1_wb<Pol, N, VLOC_MINB_K1DF>);
         if (onceb) return (int)onceb;
-        k1_wb<Pol, N, VLOC_MINB_K1DF><<<dim3(t.T, (unsigned)nb, 2), kThreads, WSmem<Pol, N>::sm, st>>>(
+        return pdl_launch(k1_wb<Pol, N, VLOC_MINB_K1DF>, dim3(t.T, (unsigned)nb, 2), kThreads, WSmem<Pol, N>::sm, st,
             t, (const typename Pol::TW*)tw3, (const double2*)coeffs, (typename Pol::V*)cyl);
     } else {
         static const cudaError_t once = WSmem<Pol, N>::ensure(k1_w<Pol, N>);
         if (once) return (int)once;
-        k1_w<Pol, N><<<dim3(t.T, (unsigned)nb, 2), kThreads, WSmem<Pol, N>::sm, st>>>(
-            t, (const typename Pol::TW*)tw3, (const double2*)coeffs, (typename Pol::V*)cyl);
+        return pdl_launch(k1_w<Pol, N>, dim3(t.T, (unsigned)nb, 2), kThreads, WSmem<Pol, N>::sm, st, t, (const
+            typename Pol::TW*)tw3, (const double2*)coeffs, (typename Pol::V*)cyl);
     }
-    return (int)cudaGetLastError();
 }
 template <int P, int N>
 int LaunchF64<P, N>::k2(int sign, const DevTables& t, const void* tw2, long long nb, void* cyl, void* slab,
@@ -593,28 +601,27 @@ int LaunchF64<P, N>::k2(int sign, const DevTables& t, const void* tw2, long long
         if (sign > 0) {
             static const cudaError_t onceb = WSmem<Pol, N>::ensure(k2_wb<Pol, +1, N, VLOC_MINB_K2IDF>);
             if (onceb) return (int)onceb;
-            k2_wb<Pol, +1, N, VLOC_MINB_K2IDF><<<grid, kThreads, WSmem<Pol, N>::sm, st>>>(t, (const typename Pol::TW*)tw2, (V*)cyl,
-                                                                            (V*)slab);
+            return pdl_launch(k2_wb<Pol, +1, N, VLOC_MINB_K2IDF>, grid, kThreads, WSmem<Pol, N>::sm, st, t, (const
+                typename Pol::TW*)tw2, (V*)cyl, (V*)slab);
         } else {
             static const cudaError_t onceb = WSmem<Pol, N>::ensure(k2_wb<Pol, -1, N, VLOC_MINB_K2FDF>);
             if (onceb) return (int)onceb;
-            k2_wb<Pol, -1, N, VLOC_MINB_K2FDF><<<grid, kThreads, WSmem<Pol, N>::sm, st>>>(t, (const typename Pol::TW*)tw2, (V*)cyl,
-                                                                            (V*)slab);
+            return pdl_launch(k2_wb<Pol, -1, N, VLOC_MINB_K2FDF>, grid, kThreads, WSmem<Pol, N>::sm, st, t, (const
+                typename Pol::TW*)tw2, (V*)cyl, (V*)slab);
         }
     } else {
         if (sign > 0) {
             static const cudaError_t once = WSmem<Pol, N>::ensure(k2_w<Pol, +1, N>);
             if (once) return (int)once;
-            k2_w<Pol, +1, N><<<grid, kThreads, WSmem<Pol, N>::sm, st>>>(t, (const typename Pol::TW*)tw2, (V*)cyl,
-                                                                        (V*)slab);
+            return pdl_launch(k2_w<Pol, +1, N>, grid, kThreads, WSmem<Pol, N>::sm, st, t, (const typename
+                Pol::TW*)tw2, (V*)cyl, (V*)slab);
         } else {
             static const cudaError_t once = WSmem<Pol, N>::ensure(k2_w<Pol, -1, N>);
             if (once) return (int)once;
-            k2_w<Pol, -1, N><<<grid, kThreads, WSmem<Pol, N>::sm, st>>>(t, (const typename Pol::TW*)tw2, (V*)cyl,
-                                                                        (V*)slab);
+            return pdl_launch(k2_w<Pol, -1, N>, grid, kThreads, WSmem<Pol, N>::sm, st, t, (const typename
+                Pol::TW*)tw2, (V*)cyl, (V*)slab);
         }
     }
-    return (int)cudaGetLastError();
 }
 template <int P, int N>
 int LaunchF64<P, N>::k3(const DevTables& t, const void* tw1, const void* V, long long nb, void* slab,
@@ -628,16 +635,14 @@ int LaunchF64<P, N>::k3(const DevTables& t, const void* tw1, const void* V, long
                 sm <= 48 * 1024 ? cudaSuccess
                                 : cudaFuncSetAttribute(k3q_w<Pol, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
             if (onceq) return (int)onceq;
-            k3q_w<Pol, N><<<grid, kThreads, sm, st>>>(t, (const typename Pol::TW*)tw1, (const typename Pol::VR*)V,
-                                                      (typename Pol::V*)slab);
-            return (int)cudaGetLastError();
+            return pdl_launch(k3q_w<Pol, N>, grid, kThreads, sm, st, t, (const typename Pol::TW*)tw1, (const typename
+                Pol::VR*)V, (typename Pol::V*)slab);
         }
     }
     static const cudaError_t once = WSmem<Pol, N>::ensure(k3_w<Pol, N>);
     if (once) return (int)once;
-    k3_w<Pol, N><<<grid, kThreads, WSmem<Pol, N>::sm, st>>>(t, (const typename Pol::TW*)tw1,
-                                                           (const typename Pol::VR*)V, (typename Pol::V*)slab);
-    return (int)cudaGetLastError();
+    return pdl_launch(k3_w<Pol, N>, grid, kThreads, WSmem<Pol, N>::sm, st, t, (const typename Pol::TW*)tw1, (const
+        typename Pol::VR*)V, (typename Pol::V*)slab);
 }
 template <int P, int N>
 int LaunchF64<P, N>::k4(const DevTables& t, const void* tw3, const void* cyl, long long nb, void* out,
@@ -647,17 +652,16 @@ int LaunchF64<P, N>::k4(const DevTables& t, const void* tw3, const void* cyl, lo
     if constexpr (df_floors<Pol, N>()) {
         static const cudaError_t onceb = WSmem<Pol, N>::ensure(k4_wb<Pol, N, VLOC_MINB_K4DF>);
         if (onceb) return (int)onceb;
-        k4_wb<Pol, N, VLOC_MINB_K4DF><<<dim3(t.T, (unsigned)nb, 2), kThreads, WSmem<Pol, N>::sm, st>>>(
+        return pdl_launch(k4_wb<Pol, N, VLOC_MINB_K4DF>, dim3(t.T, (unsigned)nb, 2), kThreads, WSmem<Pol, N>::sm, st,
             t, (const typename Pol::TW*)tw3, (const typename Pol::V*)cyl, (double2*)out, scale, (const double*)diag,
             (const double2*)cin);
     } else {
         static const cudaError_t once = WSmem<Pol, N>::ensure(k4_w<Pol, N>);
         if (once) return (int)once;
-        k4_w<Pol, N><<<dim3(t.T, (unsigned)nb, 2), kThreads, WSmem<Pol, N>::sm, st>>>(
-            t, (const typename Pol::TW*)tw3, (const typename Pol::V*)cyl, (double2*)out, scale, (const double*)diag,
-            (const double2*)cin);
+        return pdl_launch(k4_w<Pol, N>, dim3(t.T, (unsigned)nb, 2), kThreads, WSmem<Pol, N>::sm, st, t, (const
+            typename Pol::TW*)tw3, (const typename Pol::V*)cyl, (double2*)out, scale, (const double*)diag, (const
+            double2*)cin);
     }
-    return (int)cudaGetLastError();
 }
 
 }  // namespace vloc

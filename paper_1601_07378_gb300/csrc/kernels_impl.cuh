@@ -21,6 +21,7 @@
 
 #include "fft_core.cuh"
 #include "internal.h"
+#include "pdl.cuh"
 
 namespace vloc {
 
@@ -117,6 +118,7 @@ __device__ __forceinline__ void rows_in(V* buf, const V* __restrict__ cb, const 
 template <typename T>
 __global__ void __launch_bounds__(kThreads) k1_scatter_zpass(DevTables t, AxisPlan az, const V2<T>* __restrict__ tw3,
                                                             const V2<T>* __restrict__ coeffs, V2<T>* __restrict__ cyl) {
+    pdl_begin();
     using V = V2<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int n3 = t.n3;
@@ -161,6 +163,7 @@ template <typename T> struct SlabRows {  // all y rows of one plane's slab tile
 template <typename T, int S>
 __global__ void __launch_bounds__(kThreads) k2_ypass(DevTables t, AxisPlan ay, const V2<T>* __restrict__ tw2,
                                                     V2<T>* cyl, V2<T>* slab) {
+    pdl_begin();
     using V = V2<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int n2 = t.n2, n3 = t.n3;
@@ -210,6 +213,7 @@ template <typename T> struct TimesV {  // psi(x) * V(x, y, z) into shared memory
 template <typename T>
 __global__ void __launch_bounds__(kThreads) k3_xpass_v(DevTables t, AxisPlan ax, const V2<T>* __restrict__ tw1,
                                                       const T* __restrict__ Vr, V2<T>* slab) {
+    pdl_begin();
     using V = V2<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int n1 = t.n1, n2 = t.n2, n3 = t.n3;
@@ -238,6 +242,7 @@ template <typename T>
 __global__ void __launch_bounds__(kThreads) k4_zpass_gather(DevTables t, AxisPlan az, const V2<T>* __restrict__ tw3,
                                                            const V2<T>* __restrict__ cyl, V2<T>* out, T scale,
                                                            const T* __restrict__ diag, const V2<T>* cin) {
+    pdl_begin();
     using V = V2<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int n3 = t.n3;
@@ -463,34 +468,33 @@ template <typename T> int Launch<T>::twiddles(void* tw, int n, cudaStream_t st) 
 template <typename T>
 int Launch<T>::k1(const DevTables& t, const LaunchAxes& ax, const void* tw3, const void* coeffs, long long nb, void* cyl,
                   cudaStream_t st) {
-    k1_scatter_zpass<T><<<dim3(t.T, (unsigned)nb), kThreads, smem(t.n3), st>>>(t, axis_of(ax, 2), (const V2<T>*)tw3,
-                                                                               (const V2<T>*)coeffs, (V2<T>*)cyl);
-    return (int)cudaGetLastError();
+    return pdl_launch(k1_scatter_zpass<T>, dim3(t.T, (unsigned)nb), kThreads, smem(t.n3), st, t, axis_of(ax, 2),
+        (const V2<T>*)tw3, (const V2<T>*)coeffs, (V2<T>*)cyl);
 }
 template <typename T>
 int Launch<T>::k2(int sign, const DevTables& t, const LaunchAxes& ax, const void* tw2, long long nb, void* cyl,
                   void* slab, cudaStream_t st) {
     const dim3 grid(t.NP, (t.n3 + kLines - 1) / kLines, (unsigned)nb);
     if (sign > 0)
-        k2_ypass<T, +1><<<grid, kThreads, smem(t.n2), st>>>(t, axis_of(ax, 1), (const V2<T>*)tw2, (V2<T>*)cyl, (V2<T>*)slab);
+        return pdl_launch(k2_ypass<T, +1>, grid, kThreads, smem(t.n2), st, t, axis_of(ax, 1), (const V2<T>*)tw2,
+            (V2<T>*)cyl, (V2<T>*)slab);
     else
-        k2_ypass<T, -1><<<grid, kThreads, smem(t.n2), st>>>(t, axis_of(ax, 1), (const V2<T>*)tw2, (V2<T>*)cyl, (V2<T>*)slab);
-    return (int)cudaGetLastError();
+        return pdl_launch(k2_ypass<T, -1>, grid, kThreads, smem(t.n2), st, t, axis_of(ax, 1), (const V2<T>*)tw2,
+            (V2<T>*)cyl, (V2<T>*)slab);
 }
 template <typename T>
 int Launch<T>::k3(const DevTables& t, const LaunchAxes& ax, const void* tw1, const void* V, long long nb, void* slab,
                   cudaStream_t st) {
     const dim3 grid(t.n2, (t.n3 + kLines - 1) / kLines, (unsigned)nb);
-    k3_xpass_v<T><<<grid, kThreads, smem(t.n1), st>>>(t, axis_of(ax, 0), (const V2<T>*)tw1, (const T*)V, (V2<T>*)slab);
-    return (int)cudaGetLastError();
+    return pdl_launch(k3_xpass_v<T>, grid, kThreads, smem(t.n1), st, t, axis_of(ax, 0), (const V2<T>*)tw1, (const
+        T*)V, (V2<T>*)slab);
 }
 template <typename T>
 int Launch<T>::k4(const DevTables& t, const LaunchAxes& ax, const void* tw3, const void* cyl, long long nb, void* out,
                   const void* diag, const void* cin, cudaStream_t st) {
     const T scale = (T)(1.0 / ((double)t.n1 * t.n2 * t.n3));
-    k4_zpass_gather<T><<<dim3(t.T, (unsigned)nb), kThreads, smem(t.n3), st>>>(
-        t, axis_of(ax, 2), (const V2<T>*)tw3, (const V2<T>*)cyl, (V2<T>*)out, scale, (const T*)diag, (const V2<T>*)cin);
-    return (int)cudaGetLastError();
+    return pdl_launch(k4_zpass_gather<T>, dim3(t.T, (unsigned)nb), kThreads, smem(t.n3), st, t, axis_of(ax, 2),
+        (const V2<T>*)tw3, (const V2<T>*)cyl, (V2<T>*)out, scale, (const T*)diag, (const V2<T>*)cin);
 }
 template <typename T>
 int Launch<T>::k3b(const DevTables& t, const LaunchAxes& ax, const void* tw1, const void* sc, const void* sg,

@@ -1,6 +1,7 @@
 // kernels_line.cu -- dispatch of the line path (kernels_line.h) and the
 // transpose of V that its y/x pass reads.
 #include "kernels_line.h"
+#include "pdl.cuh"
 
 namespace vloc {
 namespace line {
@@ -42,6 +43,7 @@ bool z_length(int n3) {
 // 32 x 32 tiles of (y, z) at one x through shared memory, so that both sides
 // are coalesced; 7 MB of traffic at 96^3 (about 3 us), once per call.
 __global__ void __launch_bounds__(256) k_vt(const float* __restrict__ V, float* __restrict__ VT, int n2, int n3) {
+    pdl_begin();
     __shared__ float tile[32][33];
     const int z0 = blockIdx.x * 32, y0 = blockIdx.y * 32, x = blockIdx.z, n1 = gridDim.z;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -52,8 +54,7 @@ __global__ void __launch_bounds__(256) k_vt(const float* __restrict__ V, float* 
         if (z0 + j < n3 && y0 + tx < n2) VT[((long long)(z0 + j) * n1 + x) * n2 + y0 + tx] = tile[tx][j];
 }
 int launch_vt(const float* V, float* VT, const Tables& t, cudaStream_t st) {
-    k_vt<<<dim3((t.n3 + 31) / 32, (t.n2 + 31) / 32, t.n1), 256, 0, st>>>(V, VT, t.n2, t.n3);
-    return (int)cudaGetLastError();
+    return pdl_launch(k_vt, dim3((t.n3 + 31) / 32, (t.n2 + 31) / 32, t.n1), 256, 0, st, V, VT, t.n2, t.n3);
 }
 
 #define VLOC_CASE_INV(N) case N: return LaunchZ<N>::inv(t, tw3, c, nb, nreal, D, st);
@@ -91,6 +92,7 @@ int launch_dens(const Tables& t, const float2* D, long long nb, int bpg, const f
 // written along z.  Sum over the groups as in k_reduce_partials_f32.
 __global__ void __launch_bounds__(256) k_dens_reduce(const float* __restrict__ partial, int ng, int n2, int n3,
                                                      double* __restrict__ acc, int first, float* __restrict__ out) {
+    pdl_begin();
     __shared__ float ts[32][33], tc[32][33];
     const int z0 = blockIdx.x * 32, y0 = blockIdx.y * 32, x = blockIdx.z, n1 = gridDim.z;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -122,8 +124,8 @@ __global__ void __launch_bounds__(256) k_dens_reduce(const float* __restrict__ p
 }
 int launch_dens_reduce(const Tables& t, const float* partial, int ng, double* acc, int first, float* out,
                        cudaStream_t st) {
-    k_dens_reduce<<<dim3((t.n3 + 31) / 32, (t.n2 + 31) / 32, t.n1), 256, 0, st>>>(partial, ng, t.n2, t.n3, acc, first, out);
-    return (int)cudaGetLastError();
+    return pdl_launch(k_dens_reduce, dim3((t.n3 + 31) / 32, (t.n2 + 31) / 32, t.n1), 256, 0, st, partial, ng, t.n2,
+        t.n3, acc, first, out);
 }
 int launch_yx(const Tables& t, const float2* tw2, const float* VT, long long nb, float2* D, cudaStream_t st) {
 #define VLOC_CASE0(N) case N: return LaunchYX<0, N>::run(t, tw2, VT, nb, D, st);

@@ -24,6 +24,7 @@
 #include "fft_core.cuh"
 #include "kernels_line.h"
 #include "line_dft.cuh"
+#include "pdl.cuh"
 
 namespace vloc {
 namespace line {
@@ -224,6 +225,7 @@ template <class C, int N2> __device__ __forceinline__ void yx_thin(bool fwd, con
 template <int CLS, int N1, int N2>
 __global__ void __launch_bounds__(64 * YX<CLS, N1, N2>::PAIRS, YX<CLS, N1, N2>::MINB)
     kl_yx(Tables t, const float2* __restrict__ tw2, const float* __restrict__ VT, int nb, int bpc, float2* D) {
+    pdl_begin();
     using C = YX<CLS, N1, N2>;
     constexpr int NBB = C::NBB;
     const int z = blockIdx.x;
@@ -270,9 +272,8 @@ int launch_yx_n(const Tables& t, const float2* tw2, const float* VT, long long n
     // 1.59 at 128^3), but few enough that the grid is four waves deep
     int bpc = C::NBB == 2 && N2 % 32 == 0 ? 8 : 4;
     while (bpc > C::NBB && (long long)t.n3 * ((nb + bpc - 1) / bpc) < 152ll * C::MINB * 4) bpc /= 2;
-    kl_yx<CLS, N1, N2><<<dim3(t.n3, (unsigned)((nb + bpc - 1) / bpc)), 64 * C::PAIRS, C::smem, st>>>(t, tw2, VT, (int)nb,
-                                                                                                  bpc, D);
-    return (int)cudaGetLastError();
+    return pdl_launch(kl_yx<CLS, N1, N2>, dim3(t.n3, (unsigned)((nb + bpc - 1) / bpc)), 64 * C::PAIRS, C::smem, st,
+        t, tw2, VT, (int)nb, bpc, D);
 }
 // n1 = N1, every n2 of the class
 template <int CLS, int N1>

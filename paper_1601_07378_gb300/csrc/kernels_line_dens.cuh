@@ -28,6 +28,7 @@ template <int CLS, int N1, int N2>
 __global__ void __launch_bounds__(64 * YXD<CLS, N1, N2>::PAIRS, YXD<CLS, N1, N2>::MINB)
     kl_dens(Tables t, const float2* __restrict__ D, int nb, int bpg, const float* __restrict__ occ, long long b_base,
             int pair_mode, long long nreal, float* __restrict__ partial) {
+    pdl_begin();
     using C = YXD<CLS, N1, N2>;
     constexpr int M = N1 / 2, Q = N1 / 4, AP = C::AP;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -78,9 +79,8 @@ int launch_dens_n(const Tables& t, const float2* D, long long nb, int bpg, const
     using C = YXD<CLS, N1, N2>;
     static const cudaError_t once = line_smem(kl_dens<CLS, N1, N2>, C::smem);
     if (once) return (int)once;
-    kl_dens<CLS, N1, N2><<<dim3(t.n3, (unsigned)((nb + bpg - 1) / bpg)), 64 * C::PAIRS, C::smem, st>>>(
+    return pdl_launch(kl_dens<CLS, N1, N2>, dim3(t.n3, (unsigned)((nb + bpg - 1) / bpg)), 64 * C::PAIRS, C::smem, st,
         t, D, (int)nb, bpg, occ, b_base, pair, nreal, partial);
-    return (int)cudaGetLastError();
 }
 template <int CLS, int N1>
 int LaunchDens<CLS, N1>::run(const Tables& t, const float2* D, long long nb, int bpg, const float* occ, long long b_base,

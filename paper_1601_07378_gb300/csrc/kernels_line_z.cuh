@@ -52,6 +52,7 @@ template <int N, int MODE>
 __global__ void __launch_bounds__(kThreads, minb_k1(N)) kl_z_inv(Tables t, const float2* __restrict__ tw3,
                                                             const float2* __restrict__ coeffs, long long nreal,
                                                             float2* __restrict__ D) {
+    pdl_begin();
     using SC = Sched<N>;
     static_assert(SC::nst == 2, "quarter-band z-pass: two-stage lengths");
     using QR = QRows<N>;
@@ -160,6 +161,7 @@ template <int N, bool GM>
 __global__ void __launch_bounds__(kThreads, GM ? minb_k4q(N, true) : minb_k4d(N))
     kl_z_fwd(Tables t, const float2* __restrict__ tw3, const float2* __restrict__ D, long long nreal, float2* out,
              float scale, const float* __restrict__ diag, const float2* cin) {
+    pdl_begin();
     using SC = Sched<N>;
     static_assert(SC::nst == 2, "quarter-band z-pass: two-stage lengths");
     using QR = QRows<N>;
@@ -244,8 +246,7 @@ int launch_z_inv_n(const Tables& t, const float2* tw3, const float2* c, long lon
                    cudaStream_t st) {
     static const cudaError_t once = CtSmem<N>::ensure(kl_z_inv<N, MODE>);
     if (once) return (int)once;
-    kl_z_inv<N, MODE><<<dim3(t.G, (unsigned)nb), kThreads, CtSmem<N>::sm, st>>>(t, tw3, c, nreal, D);
-    return (int)cudaGetLastError();
+    return pdl_launch(kl_z_inv<N, MODE>, dim3(t.G, (unsigned)nb), kThreads, CtSmem<N>::sm, st, t, tw3, c, nreal, D);
 }
 template <int N>
 int LaunchZ<N>::inv(const Tables& t, const float2* tw3, const float2* c, long long nb, long long nreal, float2* D,
@@ -260,8 +261,8 @@ int launch_z_fwd_n(const Tables& t, const float2* tw3, const float2* D, long lon
     static const cudaError_t once = CtSmem<N>::ensure(kl_z_fwd<N, GM>);
     if (once) return (int)once;
     const float scale = (float)(1.0 / ((double)t.n1 * t.n2 * t.n3));
-    kl_z_fwd<N, GM><<<dim3(t.G, (unsigned)nb), kThreads, CtSmem<N>::sm, st>>>(t, tw3, D, nreal, out, scale, diag, c);
-    return (int)cudaGetLastError();
+    return pdl_launch(kl_z_fwd<N, GM>, dim3(t.G, (unsigned)nb), kThreads, CtSmem<N>::sm, st, t, tw3, D, nreal, out,
+        scale, diag, c);
 }
 template <int N>
 int LaunchZ<N>::fwd(const Tables& t, const float2* tw3, const float2* D, long long nb, long long nreal, float2* out,

@@ -1,0 +1,43 @@
+// pdl.cuh -- programmatic dependent launch of the chain's kernels.
+//
+// The passes of an apply are short dependent launches on one stream (5 to 10 us
+// each for a few bands), so the launch latency between them counts.  A kernel
+// launched by pdl_launch() may be set up while its predecessor in the stream
+// drains; it must start with pdl_begin(), which waits until everything before
+// it has completed and is visible, before it touches memory.  (A kernel that
+// begins so may also be launched the ordinary way.)  No kernel triggers its
+// successor early: blocks that wait take their place on the SMs unevenly while
+// the predecessor runs, which measured slower everywhere (below: GPU time per
+// apply in us without the attribute / early trigger / as it is).
+//   FP32  24^3 x 1  21.7 / 12.5 / 11.7    96^3 x 8   53.3 / 41.6 / 35.9
+//         48^3 x 20 32.9 / 20.6 / 16.4    96^3 x 512 1900 / 1726 / 1613
+//   (the first column: the five-launch chain, the others the line path)
+//   FP64  24^3 x 1  34.9 / 25.4 / 24.7    48^3 x 4   80 / 87 to 156 / 69
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include <utility>
+
+namespace vloc {
+
+__device__ __forceinline__ void pdl_begin() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <class... P, class... A>
+inline int pdl_launch(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, A&&... args) {
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, P(std::forward<A>(args))...);
+    if (e != cudaSuccess) cudaGetLastError();  // reported here, not by a later check
+    return (int)e;
+}
+
+}  // namespace vloc
