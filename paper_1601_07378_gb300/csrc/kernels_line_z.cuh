@@ -46,6 +46,22 @@ template <bool GM> __device__ __forceinline__ bool dense_rows(const Tables& t, i
     return pa >= 0 || pb >= 0;
 }
 
+// Lane -> (line pair, unit) of the stages that meet the caller's arrays (the
+// inverse's first, the forward's last).  ED (caller lists in stick order): a warp
+// takes 8 line pairs and 4 consecutive units instead of 16 and 2, so that an
+// access covers 32 bytes of each stick's run; these accesses are most of a
+// block's load/store wavefronts.  96^3 x 1024 bands: inverse 0.452 -> 0.449 ms,
+// forward 0.432 -> 0.424; 128^3 x 256: 0.263 -> 0.263, 0.267 -> 0.261.  Lists in
+// another order have no runs to cover and lose rows of the table that two units
+// share (shuffled, 96^3: 0.653 -> 0.673, 0.516 -> 0.524), so they keep 16 and 2.
+template <bool ED> __device__ __forceinline__ int edge_slot() {
+    return ED ? (threadIdx.x & 7) + ((threadIdx.x >> 5) & 1) * 8 : slot_of();
+}
+template <bool ED> __device__ __forceinline__ int edge_unit() {
+    return ED ? ((threadIdx.x >> 3) & 3) + (threadIdx.x >> 6) * 4 : 2 * warp_of() + sub_of();
+}
+static_assert(kWarps % 2 == 0, "edge mapping: warps in pairs");
+
 // MODE 0: first-stage inputs through the group's dense table, 1: addressed
 // from the sticks' runs (caller lists in stick order), 2: Gamma-point pairs.
 template <int N, int MODE>
@@ -69,9 +85,10 @@ __global__ void __launch_bounds__(kThreads, minb_k1(N)) kl_z_inv(Tables t, const
     SmemP sb{buf};
     if constexpr (MODE < 2) {
         const float2* c = coeffs + b * t.npw;
+        const int slot = edge_slot<MODE == 1>();
 #pragma unroll
         for (int u = 0; u < UA; ++u) {
-            const int i = 2 * (warp + u * W) + sub;
+            const int i = edge_unit<MODE == 1>() + 2 * W * u;
             if (NA % (2 * W) == 0 || i < NA) {
                 P2f h[R0];
                 if constexpr (MODE == 1) {
@@ -156,8 +173,8 @@ __global__ void __launch_bounds__(kThreads, minb_k1(N)) kl_z_inv(Tables t, const
 // Forward: first stage (reversed schedule) straight from the dense rows; the
 // last one stores each result to its caller position through the dense table
 // or (Gamma) leaves it in the tile for the gather that separates the
-// pairs; times 1/N, plus diag times the band.
-template <int N, bool GM>
+// pairs; times 1/N, plus diag times the band.  ED: see edge_slot.
+template <int N, bool GM, bool ED>
 __global__ void __launch_bounds__(kThreads, GM ? minb_k4q(N, true) : minb_k4d(N))
     kl_z_fwd(Tables t, const float2* __restrict__ tw3, const float2* __restrict__ D, long long nreal, float2* out,
              float scale, const float* __restrict__ diag, const float2* cin) {
@@ -181,13 +198,14 @@ __global__ void __launch_bounds__(kThreads, GM ? minb_k4q(N, true) : minb_k4d(N)
     load_tw<float>(stw, tw3, N);
     __syncthreads();
     if constexpr (!GM) {
-        if (!act) return;
+        if (!ED && !act) return;  // ED: `act` is not this lane's line pair; the table's -1 drops absent ones
+        const int slot = edge_slot<ED>();
         const int* zd = t.zd + (size_t)g * (QR::groups() * NA) * 32 + 2 * slot;
         float2* o = out + b * t.npw;
         const float2* ci = diag ? cin + b * t.npw : cin;
 #pragma unroll
         for (int u = 0; u < L::U; ++u) {
-            const int i = 2 * (warp + u * W) + sub;
+            const int i = edge_unit<ED>() + 2 * W * u;
             if (L::NI % (2 * W) == 0 || i < L::NI) {
                 int2 e[R0];
                 sfor<R0>([&](auto rc) {
@@ -255,20 +273,21 @@ int LaunchZ<N>::inv(const Tables& t, const float2* tw3, const float2* c, long lo
            : t.runs ? launch_z_inv_n<N, 1>(t, tw3, c, nb, nreal, D, st)
                     : launch_z_inv_n<N, 0>(t, tw3, c, nb, nreal, D, st);
 }
-template <int N, bool GM>
+template <int N, bool GM, bool ED>
 int launch_z_fwd_n(const Tables& t, const float2* tw3, const float2* D, long long nb, long long nreal, float2* out,
                    const float* diag, const float2* c, cudaStream_t st) {
-    static const cudaError_t once = CtSmem<N>::ensure(kl_z_fwd<N, GM>);
+    static const cudaError_t once = CtSmem<N>::ensure(kl_z_fwd<N, GM, ED>);
     if (once) return (int)once;
     const float scale = (float)(1.0 / ((double)t.n1 * t.n2 * t.n3));
-    return pdl_launch(kl_z_fwd<N, GM>, dim3(t.G, (unsigned)nb), kThreads, CtSmem<N>::sm, st, t, tw3, D, nreal, out,
+    return pdl_launch(kl_z_fwd<N, GM, ED>, dim3(t.G, (unsigned)nb), kThreads, CtSmem<N>::sm, st, t, tw3, D, nreal, out,
         scale, diag, c);
 }
 template <int N>
 int LaunchZ<N>::fwd(const Tables& t, const float2* tw3, const float2* D, long long nb, long long nreal, float2* out,
                     const float* diag, const float2* c, cudaStream_t st) {
-    return t.gamma ? launch_z_fwd_n<N, true>(t, tw3, D, nb, nreal, out, diag, c, st)
-                   : launch_z_fwd_n<N, false>(t, tw3, D, nb, nreal, out, diag, c, st);
+    return t.gamma  ? launch_z_fwd_n<N, true, false>(t, tw3, D, nb, nreal, out, diag, c, st)
+           : t.runs ? launch_z_fwd_n<N, false, true>(t, tw3, D, nb, nreal, out, diag, c, st)
+                    : launch_z_fwd_n<N, false, false>(t, tw3, D, nb, nreal, out, diag, c, st);
 }
 
 }  // namespace line
