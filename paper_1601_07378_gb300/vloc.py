@@ -9,6 +9,7 @@ raises.
 from __future__ import annotations
 
 import ctypes
+import math
 import os
 import threading
 
@@ -148,14 +149,19 @@ def _check(code: int, what: str):
         raise VlocError(code, what)
 
 
-def _stream_ptr(stream=None):
+# The marshalling below runs on every call, and a call on a few bands is only
+# some 10 us of GPU time: device addresses and the stream go through ctypes as
+# plain integers (the argument types are set once in ``load``), and what depends
+# on the plan alone is worked out when it is made.
+def _stream_ptr(stream=None) -> int:
+    if stream is not None:
+        return stream.cuda_stream
     import torch
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
-def _ptr(t) -> ctypes.c_void_p:
-    return ctypes.c_void_p(t.data_ptr())
+def _ptr(t) -> int:
+    return t.data_ptr()
 
 
 PEAK_KINDS = {"dfma": 0, "dadd": 1, "ffma": 2, "ffma2": 3, "fadd2": 4}
@@ -199,6 +205,7 @@ class VlocPlan:
             raise TypeError("dtype must be torch.complex64 or torch.complex128")
         self.lib = load()
         self.grid = tuple(int(x) for x in grid)
+        self.ngrid = math.prod(self.grid)
         self.dtype = dtype
         self.real_dtype = torch.float32 if dtype == torch.complex64 else torch.float64
         g = np.ascontiguousarray(np.asarray(glist, dtype=np.int32).reshape(-1, 3))
@@ -227,7 +234,7 @@ class VlocPlan:
         if poison:
             flags |= VLOC_POISON_WORKSPACE
         h = ctypes.c_void_p()
-        sp = ctypes.c_void_p(None) if host_only else _stream_ptr(stream)
+        sp = None if host_only else _stream_ptr(stream)
         _check(self.lib.vloc_plan_create(ctypes.byref(h), *self.grid,
                                          g.ctypes.data_as(ctypes.POINTER(ctypes.c_int32)), self.npw,
                                          flags, int(chunk), sp), "vloc_plan_create")
@@ -317,8 +324,8 @@ class VlocPlan:
             raise ValueError(f"{name} last dim must be npw={self.npw}")
 
     def _check_V(self, V):
-        if not V.is_cuda or V.dtype != self.real_dtype or not V.is_contiguous() or V.numel() != np.prod(self.grid):
-            raise ValueError(f"V must be a contiguous CUDA {self.real_dtype} tensor with {np.prod(self.grid)} elements")
+        if not V.is_cuda or V.dtype != self.real_dtype or not V.is_contiguous() or V.numel() != self.ngrid:
+            raise ValueError(f"V must be a contiguous CUDA {self.real_dtype} tensor with {self.ngrid} elements")
 
     def _check_out(self, out, c, name="out"):
         # the kernels write as many bands as they read: a smaller buffer would be overrun
@@ -329,10 +336,10 @@ class VlocPlan:
     # ---------------------------------------------------------------- calls
     def apply(self, c, V, out=None, *, adjoint: bool = False, stream=None):
         """out = A c (or A^H c) for c of shape [..., npw]."""
-        import torch
         self._check_c(c)
         self._check_V(V)
         if out is None:
+            import torch
             out = torch.empty_like(c)
         else:
             self._check_out(out, c)
@@ -344,12 +351,12 @@ class VlocPlan:
 
     def apply_h(self, c, V, diag, out=None, *, stream=None):
         """out = (diag(d) + A) c: V_loc plus a term diagonal in G (e.g. kinetic |k+G|^2/2)."""
-        import torch
         self._check_c(c)
         self._check_V(V)
         if not diag.is_cuda or diag.dtype != self.real_dtype or not diag.is_contiguous() or diag.numel() != self.npw:
             raise ValueError(f"diag must be a contiguous CUDA {self.real_dtype} tensor of npw={self.npw} entries")
         if out is None:
+            import torch
             out = torch.empty_like(c)
         else:
             self._check_out(out, c)
@@ -380,7 +387,7 @@ class VlocPlan:
         if psi is None:
             psi = torch.empty((nb, *self.grid), dtype=self.dtype, device=c.device)
         elif not psi.is_cuda or psi.dtype != self.dtype or not psi.is_contiguous() or \
-                psi.numel() != nb * int(np.prod(self.grid)):
+                psi.numel() != nb * self.ngrid:
             raise ValueError("psi must be a contiguous CUDA tensor of nb full grids")
         _check(self.lib.vloc_to_real(self.handle, _ptr(c), nb, _ptr(psi), _stream_ptr(stream)), "vloc_to_real")
         return psi
@@ -388,7 +395,7 @@ class VlocPlan:
     def to_recip(self, u, out=None, *, stream=None):
         """out_n(G) = (1/N) sum_r u_n(r) exp(-2 pi i G.r/n) for full grids u [nb, n1, n2, n3]."""
         import torch
-        N = int(np.prod(self.grid))
+        N = self.ngrid
         if not u.is_cuda or u.dtype != self.dtype or not u.is_contiguous() or u.numel() % N:
             raise ValueError("u must be a contiguous CUDA tensor of full grids")
         nb = u.numel() // N
@@ -412,8 +419,8 @@ class VlocPlan:
         if rho is None:
             rho = torch.empty(self.grid, dtype=self.real_dtype, device=c.device)
         elif not rho.is_cuda or rho.dtype != self.real_dtype or not rho.is_contiguous() or \
-                rho.numel() != int(np.prod(self.grid)):
-            raise ValueError(f"rho must be a contiguous CUDA {self.real_dtype} tensor with {np.prod(self.grid)} elements")
+                rho.numel() != self.ngrid:
+            raise ValueError(f"rho must be a contiguous CUDA {self.real_dtype} tensor with {self.ngrid} elements")
         _check(self.lib.vloc_density(self.handle, _ptr(c), _ptr(occ) if occ is not None else None, nb, _ptr(rho),
                                      _stream_ptr(stream)), "vloc_density")
         return rho
@@ -428,7 +435,7 @@ class VlocPlan:
             raise ValueError("apply_host takes CPU tensors")
         if c_host.dtype != self.dtype or not c_host.is_contiguous() or c_host.shape[-1] != self.npw:
             raise ValueError("bad host coefficients")
-        if V_host.dtype != self.real_dtype or not V_host.is_contiguous() or V_host.numel() != np.prod(self.grid):
+        if V_host.dtype != self.real_dtype or not V_host.is_contiguous() or V_host.numel() != self.ngrid:
             raise ValueError("bad host V")
         if out_host is None:
             out_host = torch.empty_like(c_host, pin_memory=c_host.is_pinned())
