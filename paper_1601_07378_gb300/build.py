@@ -1,9 +1,9 @@
 """Build the sm_103a shared library libvloc.so in-tree (no cmake, no pip).
 
-The translation units of ``csrc/`` (the compile-time-length FP32 and
-double-float kernels split over three files each, one per precision for the
-runtime-radix kernels, the dispatch, the plan and the no-alloc entry) are compiled in parallel with
-nvcc and linked into ``paper_1601_07378_gb300/_build/libvloc.so``
+The translation units of ``csrc/`` (the compile-time-length kernels split by
+lengths into files of about the same compile time, one file per precision for
+the runtime-radix kernels, the dispatch, the plan and the no-alloc entry) are
+compiled in parallel with nvcc and linked into ``paper_1601_07378_gb300/_build/libvloc.so``
 against the shared CUDA runtime, so the library shares the runtime PyTorch
 already loaded.  ``python -m paper_1601_07378_gb300.build`` rebuilds it.
 """
@@ -21,10 +21,10 @@ LIB = os.path.join(BUILD, "libvloc.so")
 ROOT = os.path.dirname(HERE)
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-SOURCES = ["kernels_ct_a.cu", "kernels_ct_b.cu", "kernels_ct_c.cu", "kernels_df_a.cu", "kernels_df_b.cu",
-           "kernels_df_c.cu", "kernels_line.cu", *(f"kernels_line_yx{u}.cu" for u in "kjihgfedcba"),
+SOURCES = ["kernels_ct_a.cu", "kernels_ct_b.cu", "kernels_ct_c.cu", *(f"kernels_df_{u}.cu" for u in "cedfba"),
+           "kernels_line.cu", *(f"kernels_line_yx{u}.cu" for u in "kjihgfedcba"),
            *(f"kernels_line_z{u}.cu" for u in "dcba"), *(f"kernels_line_d{u}.cu" for u in "dcba"),
-            "kernels_f32.cu", "kernels_f64.cu", "kernels.cu", "plan.cpp", "noalloc.cu", "peaks.cu"]
+           "kernels_f32.cu", "kernels_f64.cu", "kernels.cu", "plan.cpp", "noalloc.cu", "peaks.cu"]
 
 
 def _cuda_home() -> str:

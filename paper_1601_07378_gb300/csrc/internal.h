@@ -34,6 +34,9 @@ struct DevTables {
     // 1 when every plane wave has l mod n3 in 0..n3/4 or n3 - n3/4 .. n3 - 1
     // (|l| <= n3/4): the z-pass kernels then skip the rows outside that band
     int zq;
+    // 1 when every stick has k mod n2 in 0..n2/4 or n2 - n2/4 .. n2 - 1: the
+    // same for the inverse y-passes of FP64-data plans
+    int yq;
     // Gamma-point plans whose every G shares a z-pass tile with its -G (gok):
     // per tile [gamma_h_ptr[t], gamma_h_ptr[t+1]) of gamma_h = {h, position
     // of G, position of -G, 0} for the half-list plane waves h whose G lies
@@ -236,6 +239,7 @@ struct HostTableLayout {
     int S, T, NP;
     int xq;  // DevTables::xq
     int zq;  // DevTables::zq
+    int yq;  // DevTables::yq
     int gok;  // DevTables::gok
     size_t o_ghp, o_gh, o_zd, o_zs, o_rn;
     int zd_rows;

@@ -263,7 +263,15 @@ __global__ void __launch_bounds__(kThreads, MINB) k1d_wb(DevTables t, const type
 }
 
 // ------------------------------------------------------------------ K2
-template <class Pol, int S, int N>
+// Q: the quarter-band form of the inverse (two-stage lengths, every stick within
+// n2/4 of k = 0).  Row r of unit i of the first stage is y = i + r NA, the rows
+// of the x-pass (QRows); those outside the band are neither looked up nor
+// transformed.  The pass is bound by the FP64 (native) or FP32 (double-float)
+// instructions that this saves: 1.144 -> 1.045 ms (native, 64^3 x 256 bands),
+// 0.622 -> 0.589 (double-float, 96^3 x 256), 0.358 -> 0.348 (72^3 x 256).  The
+// forward pass keeps every output: pruned it needs the reversed schedule, which
+// measured 1.092 against 1.063 ms, 0.657 against 0.664 and 0.370 against 0.330.
+template <class Pol, int S, int N, bool Q>
 __device__ __forceinline__ void k2w_body(const DevTables& t, const typename Pol::TW* __restrict__ tw2,
                                          typename Pol::V* cyl, typename Pol::V* slab) {
     using V = typename Pol::V;
@@ -285,24 +293,50 @@ __device__ __forceinline__ void k2w_body(const DevTables& t, const typename Pol:
     CylRowsD<V> cr{cyl + b * (long long)t.S * n3, rowmap, n3, z0};
     SlabRowsD<V> sr{slab + ((b * t.NP + plane) * (long long)N) * n3 + z0, n3};
     const bool act = slot_of_df() < lines;
-    if constexpr (S > 0)
+    if constexpr (Q) {
+        static_assert(S > 0, "inverse only");
+        using QR = QRows<N>;
+        constexpr int R0 = QR::R0, NA = QR::NA, W = kWarps;
+        constexpr int UA = (NA + 2 * W - 1) / (2 * W);
+        const int slot = slot_of_df(), sub = sub_of_df(), warp = warp_of_df();
+        SmemT<V> sb{buf};
+        if (act) {
+#pragma unroll
+            for (int u = 0; u < UA; ++u) {
+                const int i = 2 * (warp + u * W) + sub;
+                if (NA % (2 * W) == 0 || i < NA) {
+                    V h[R0];
+                    sfor<R0>([&](auto rc) {
+                        constexpr int r = decltype(rc)::value;
+                        if constexpr (QR::kind(r) == 0) h[r] = czero<V>();
+                        else h[r] = cr(i + r * NA, slot);
+                    });
+                    DftZ<R0, +1, QR::mask()>::run(h);
+#pragma unroll
+                    for (int r = 0; r < R0; ++r) sb(i * R0 + r, slot, h[r]);
+                }
+            }
+        }
+        __syncthreads();
+        NatStage<N, +1, W, 1, V, TW>::template run<false>(stw, sb, sr, slot, sub, warp, act);
+    } else if constexpr (S > 0)
         fft_ct<N, +1, kWarps, false, false, false, V, TW>(stw, cr, sr, buf, slot_of_df(), sub_of_df(), warp_of_df(),
                                                              act);
     else
         fft_ct<N, -1, kWarps, false, false, false, V, TW>(stw, sr, cr, buf, slot_of_df(), sub_of_df(), warp_of_df(),
                                                              act);
 }
-template <class Pol, int S, int N>
+template <class Pol, int S, int N, bool Q>
 __global__ void __launch_bounds__(kThreads) k2_w(DevTables t, const typename Pol::TW* __restrict__ tw2,
                                                 typename Pol::V* cyl, typename Pol::V* slab) {
     pdl_begin();
-    k2w_body<Pol, S, N>(t, tw2, cyl, slab);
+    k2w_body<Pol, S, N, Q>(t, tw2, cyl, slab);
 }
-template <class Pol, int S, int N, int MINB>
+template <class Pol, int S, int N, bool Q, int MINB>
 __global__ void __launch_bounds__(kThreads, MINB) k2_wb(DevTables t, const typename Pol::TW* __restrict__ tw2,
                                                        typename Pol::V* cyl, typename Pol::V* slab) {
     pdl_begin();
-    k2w_body<Pol, S, N>(t, tw2, cyl, slab);
+    k2w_body<Pol, S, N, Q>(t, tw2, cyl, slab);
 }
 
 // ------------------------------------------------------------------ K3
@@ -493,7 +527,11 @@ __global__ void __launch_bounds__(kThreads) k3q_w(DevTables t, const typename Po
 }
 
 // ------------------------------------------------------------------ K4
-template <class Pol, int N>
+// Q: every l in the quarter band; the transform runs in the reversed schedule,
+// whose last stage (radix R0) never forms the rows outside the band: 0.466 ->
+// 0.447 ms (native, 64^3 x 256 bands), 0.463 -> 0.448 (double-float, 96^3 x 256),
+// 0.268 -> 0.258 (72^3 x 256).
+template <class Pol, int N, bool Q>
 __device__ __forceinline__ void k4w_body(const DevTables& t, const typename Pol::TW* __restrict__ tw3,
                                          const typename Pol::V* __restrict__ cyl, double2* out, double scale,
                                          const double* __restrict__ diag, const double2* cin) {
@@ -515,8 +553,33 @@ __device__ __forceinline__ void k4w_body(const DevTables& t, const typename Pol:
         for (int z = lane; z < N; z += 32) w_at<V>(buf, z, l) = row[z];
     }
     __syncthreads();
-    fft_ct<N, -1, kWarps, false, true, true, V, TW>(stw, SmemT<V>{buf}, SmemT<V>{buf}, buf, slot_of_df(),
-                                                       sub_of_df(), warp_of_df(), slot_of_df() < lines);
+    if constexpr (Q) {
+        using QR = QRows<N>;
+        using L = RevStage<N, -1, kWarps, 1, V, TW>;
+        const int slot = slot_of_df(), sub = sub_of_df(), warp = warp_of_df();
+        const bool act = slot < lines;
+        SmemT<V> sb{buf};
+        RevStage<N, -1, kWarps, 0, V, TW>::template run<true>(stw, sb, sb, slot, sub, warp, act);
+        __syncthreads();
+        V h[L::U][QR::R0];
+        if (act) L::compute(h, stw, sb, slot, sub, warp);
+        __syncthreads();
+        if (act) {
+#pragma unroll
+            for (int u = 0; u < L::U; ++u) {
+                const int i = 2 * (warp + u * kWarps) + sub;
+                if (L::NI % (2 * kWarps) == 0 || i < L::NI) {
+                    sfor<QR::R0>([&](auto rc) {
+                        constexpr int r = decltype(rc)::value;
+                        if constexpr (QR::kind(r) != 0) sb(i + r * QR::NA, slot, h[u][r]);
+                    });
+                }
+            }
+        }
+    } else {
+        fft_ct<N, -1, kWarps, false, true, true, V, TW>(stw, SmemT<V>{buf}, SmemT<V>{buf}, buf, slot_of_df(),
+                                                           sub_of_df(), warp_of_df(), slot_of_df() < lines);
+    }
     __syncthreads();
     double2* o = out + b * t.npw;
     const double2* ci = diag ? cin + b * t.npw : cin;
@@ -535,20 +598,20 @@ __device__ __forceinline__ void k4w_body(const DevTables& t, const typename Pol:
     }
 }
 
-template <class Pol, int N>
+template <class Pol, int N, bool Q>
 __global__ void __launch_bounds__(kThreads) k4_w(DevTables t, const typename Pol::TW* __restrict__ tw3,
                                                 const typename Pol::V* __restrict__ cyl, double2* out, double scale,
                                                 const double* __restrict__ diag, const double2* cin) {
     pdl_begin();
-    k4w_body<Pol, N>(t, tw3, cyl, out, scale, diag, cin);
+    k4w_body<Pol, N, Q>(t, tw3, cyl, out, scale, diag, cin);
 }
-template <class Pol, int N, int MINB>
+template <class Pol, int N, bool Q, int MINB>
 __global__ void __launch_bounds__(kThreads, MINB) k4_wb(DevTables t, const typename Pol::TW* __restrict__ tw3,
                                                        const typename Pol::V* __restrict__ cyl, double2* out,
                                                        double scale, const double* __restrict__ diag,
                                                        const double2* cin) {
     pdl_begin();
-    k4w_body<Pol, N>(t, tw3, cyl, out, scale, diag, cin);
+    k4w_body<Pol, N, Q>(t, tw3, cyl, out, scale, diag, cin);
 }
 
 // ------------------------------------------------------------ launchers
@@ -591,37 +654,32 @@ int LaunchF64<P, N>::k1(const DevTables& t, const void* tw3, const void* coeffs,
             typename Pol::TW*)tw3, (const double2*)coeffs, (typename Pol::V*)cyl);
     }
 }
+template <class Pol, int S, int N, bool Q>
+int launch_k2w(const DevTables& t, const typename Pol::TW* tw2, long long nb, typename Pol::V* cyl,
+               typename Pol::V* slab, cudaStream_t st) {
+    const dim3 grid(t.NP, (t.n3 + kLinesDF - 1) / kLinesDF, (unsigned)nb);
+    if constexpr (df_floors<Pol, N>()) {
+        constexpr int MINB = S > 0 ? VLOC_MINB_K2IDF : VLOC_MINB_K2FDF;
+        static const cudaError_t onceb = WSmem<Pol, N>::ensure(k2_wb<Pol, S, N, Q, MINB>);
+        if (onceb) return (int)onceb;
+        return pdl_launch(k2_wb<Pol, S, N, Q, MINB>, grid, kThreads, WSmem<Pol, N>::sm, st, t, tw2, cyl, slab);
+    } else {
+        static const cudaError_t once = WSmem<Pol, N>::ensure(k2_w<Pol, S, N, Q>);
+        if (once) return (int)once;
+        return pdl_launch(k2_w<Pol, S, N, Q>, grid, kThreads, WSmem<Pol, N>::sm, st, t, tw2, cyl, slab);
+    }
+}
 template <int P, int N>
 int LaunchF64<P, N>::k2(int sign, const DevTables& t, const void* tw2, long long nb, void* cyl, void* slab,
                         cudaStream_t st) {
     using Pol = PolOf<P>;
     using V = typename Pol::V;
-    const dim3 grid(t.NP, (t.n3 + kLinesDF - 1) / kLinesDF, (unsigned)nb);
-    if constexpr (df_floors<Pol, N>()) {
-        if (sign > 0) {
-            static const cudaError_t onceb = WSmem<Pol, N>::ensure(k2_wb<Pol, +1, N, VLOC_MINB_K2IDF>);
-            if (onceb) return (int)onceb;
-            return pdl_launch(k2_wb<Pol, +1, N, VLOC_MINB_K2IDF>, grid, kThreads, WSmem<Pol, N>::sm, st, t, (const
-                typename Pol::TW*)tw2, (V*)cyl, (V*)slab);
-        } else {
-            static const cudaError_t onceb = WSmem<Pol, N>::ensure(k2_wb<Pol, -1, N, VLOC_MINB_K2FDF>);
-            if (onceb) return (int)onceb;
-            return pdl_launch(k2_wb<Pol, -1, N, VLOC_MINB_K2FDF>, grid, kThreads, WSmem<Pol, N>::sm, st, t, (const
-                typename Pol::TW*)tw2, (V*)cyl, (V*)slab);
-        }
-    } else {
-        if (sign > 0) {
-            static const cudaError_t once = WSmem<Pol, N>::ensure(k2_w<Pol, +1, N>);
-            if (once) return (int)once;
-            return pdl_launch(k2_w<Pol, +1, N>, grid, kThreads, WSmem<Pol, N>::sm, st, t, (const typename
-                Pol::TW*)tw2, (V*)cyl, (V*)slab);
-        } else {
-            static const cudaError_t once = WSmem<Pol, N>::ensure(k2_w<Pol, -1, N>);
-            if (once) return (int)once;
-            return pdl_launch(k2_w<Pol, -1, N>, grid, kThreads, WSmem<Pol, N>::sm, st, t, (const typename
-                Pol::TW*)tw2, (V*)cyl, (V*)slab);
-        }
+    const auto* tw = (const typename Pol::TW*)tw2;
+    if constexpr (Sched<N>::nst == 2) {
+        if (t.yq && sign > 0) return launch_k2w<Pol, +1, N, true>(t, tw, nb, (V*)cyl, (V*)slab, st);
     }
+    return sign > 0 ? launch_k2w<Pol, +1, N, false>(t, tw, nb, (V*)cyl, (V*)slab, st)
+                    : launch_k2w<Pol, -1, N, false>(t, tw, nb, (V*)cyl, (V*)slab, st);
 }
 template <int P, int N>
 int LaunchF64<P, N>::k3(const DevTables& t, const void* tw1, const void* V, long long nb, void* slab,
@@ -644,24 +702,35 @@ int LaunchF64<P, N>::k3(const DevTables& t, const void* tw1, const void* V, long
     return pdl_launch(k3_w<Pol, N>, grid, kThreads, WSmem<Pol, N>::sm, st, t, (const typename Pol::TW*)tw1, (const
         typename Pol::VR*)V, (typename Pol::V*)slab);
 }
+template <class Pol, int N, bool Q>
+int launch_k4w(const DevTables& t, const typename Pol::TW* tw3, const typename Pol::V* cyl, long long nb, double2* out,
+               const double* diag, const double2* cin, cudaStream_t st) {
+    const double scale = 1.0 / ((double)t.n1 * t.n2 * t.n3);
+    const dim3 grid(t.T, (unsigned)nb, 2);
+    if constexpr (df_floors<Pol, N>()) {
+        static const cudaError_t onceb = WSmem<Pol, N>::ensure(k4_wb<Pol, N, Q, VLOC_MINB_K4DF>);
+        if (onceb) return (int)onceb;
+        return pdl_launch(k4_wb<Pol, N, Q, VLOC_MINB_K4DF>, grid, kThreads, WSmem<Pol, N>::sm, st, t, tw3, cyl, out,
+                          scale, diag, cin);
+    } else {
+        static const cudaError_t once = WSmem<Pol, N>::ensure(k4_w<Pol, N, Q>);
+        if (once) return (int)once;
+        return pdl_launch(k4_w<Pol, N, Q>, grid, kThreads, WSmem<Pol, N>::sm, st, t, tw3, cyl, out, scale, diag, cin);
+    }
+}
 template <int P, int N>
 int LaunchF64<P, N>::k4(const DevTables& t, const void* tw3, const void* cyl, long long nb, void* out,
                         const void* diag, const void* cin, cudaStream_t st) {
     using Pol = PolOf<P>;
-    const double scale = 1.0 / ((double)t.n1 * t.n2 * t.n3);
-    if constexpr (df_floors<Pol, N>()) {
-        static const cudaError_t onceb = WSmem<Pol, N>::ensure(k4_wb<Pol, N, VLOC_MINB_K4DF>);
-        if (onceb) return (int)onceb;
-        return pdl_launch(k4_wb<Pol, N, VLOC_MINB_K4DF>, dim3(t.T, (unsigned)nb, 2), kThreads, WSmem<Pol, N>::sm, st,
-            t, (const typename Pol::TW*)tw3, (const typename Pol::V*)cyl, (double2*)out, scale, (const double*)diag,
-            (const double2*)cin);
-    } else {
-        static const cudaError_t once = WSmem<Pol, N>::ensure(k4_w<Pol, N>);
-        if (once) return (int)once;
-        return pdl_launch(k4_w<Pol, N>, dim3(t.T, (unsigned)nb, 2), kThreads, WSmem<Pol, N>::sm, st, t, (const
-            typename Pol::TW*)tw3, (const typename Pol::V*)cyl, (double2*)out, scale, (const double*)diag, (const
-            double2*)cin);
+    using V = typename Pol::V;
+    const auto* tw = (const typename Pol::TW*)tw3;
+    if constexpr (Sched<N>::nst == 2) {
+        if (t.zq)
+            return launch_k4w<Pol, N, true>(t, tw, (const V*)cyl, nb, (double2*)out, (const double*)diag,
+                                            (const double2*)cin, st);
     }
+    return launch_k4w<Pol, N, false>(t, tw, (const V*)cyl, nb, (double2*)out, (const double*)diag,
+                                     (const double2*)cin, st);
 }
 
 }  // namespace vloc

@@ -754,6 +754,11 @@ int vloc_plan_create(vloc_plan* out, int n1, int n2, int n3, const int32_t* g, i
             zq = z <= Q3 || z >= n3 - Q3;
         }
         L.zq = zq ? 1 : 0;
+        // and every stick within the quarter band of n2 (the inverse y-pass)
+        const int Q2 = n2 / 4;
+        bool yq = Q2 >= 1 && std::getenv("VLOC_NO_XQ") == nullptr;
+        for (int s = 0; yq && s < S; ++s) yq = stick_row[s] <= Q2 || stick_row[s] >= n2 - Q2;
+        L.yq = yq ? 1 : 0;
     }
 
     if (host_only) {
@@ -1730,6 +1735,7 @@ DevTables vloc::device_tables(const int* base, const HostTableLayout& L, int n1,
     t.n1 = n1; t.n2 = n2; t.n3 = n3; t.npw = npw;
     t.xq = L.xq;
     t.zq = L.zq;
+    t.yq = L.yq;
     t.gok = L.gok;
     t.zd_rows = L.zd_rows;
     t.zdense = base + L.o_zd;
