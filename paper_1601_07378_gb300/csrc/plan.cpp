@@ -56,7 +56,7 @@ constexpr long long kGradBandsPerGroup = 16;
 #ifndef VLOC_STAGE_SLOTS
 #define VLOC_STAGE_SLOTS 2
 #endif
-constexpr long long kBatchBranches = 4;  // parallel branches of a batched graph  // bands per group of the dL/dV x-pass (FP32 sums)
+constexpr long long kBatchBranches = 4;  // parallel branches of a batched graph
 constexpr int kLinesPerTile = 32;
 
 bool smooth235(int n) {
@@ -1458,6 +1458,19 @@ int vloc_density(vloc_plan p, const void* c, const void* occ, int64_t nb, void* 
     return launch(p, KK_AUX, st, [&] { return launch_finish_grad_v(dbl, p->d_acc, rho, p->N, st); });
 }
 
+// Whether an instance of a batch should not share the GPU with another length's
+// y/x pass.  Two such kernels on an SM evict each other's code from its
+// instruction cache: eight cubes 48^3..144^3 with 64..512 bands took 18.2 ms on
+// parallel branches and 16.7 one after another, with 4..32 bands 1.21 and 1.14;
+// 96^3 + 100^3 x 128 1.116 / 1.055; 90^3, 96^3, 108^3 x 100 1.32 / 1.22.  It is
+// the other way round where the kernels are the same (4 x 64 bands at 144^3 3.84
+// / 3.96) or short (60^3, 64^3, 72^3 x 256 0.827 / 0.857), and where the
+// instances do not fill the GPU (eight of 96^3 x 8 0.178 / 0.236; the count is
+// bands x z rows x y columns, the eight cubes with 4..32 bands lose from 800 k on).
+static bool batch_apart(vloc_plan p, int64_t nb) {
+    return p->line_on && nb * p->n3 * p->n2 >= 400000 && p->n1 + p->n2 >= 180;
+}
+
 int vloc_apply_batched(int ninst, const vloc_plan* plans, const void* const* c, const void* const* V,
                        const int64_t* nb, void* const* out, void* stream) {
     if (ninst < 0 || (ninst > 0 && (!plans || !c || !V || !nb || !out))) return VLOC_ERR_ARG;
@@ -1477,9 +1490,11 @@ int vloc_apply_batched(int ninst, const vloc_plan* plans, const void* const* c, 
     bool all_graph = ninst > 0;
     for (int i = 0; i < ninst; ++i) all_graph = all_graph && (plans[i]->flags & VLOC_GRAPH);
     if (!all_graph) return enqueue((cudaStream_t)stream);
-    // Captured as parallel branches: instance i runs on branch (i mod K) so
+    // Captured as parallel branches: instances go round K branches so
     // independent instances (each with its own workspace) overlap and fill
     // one another's kernel tails; instances sharing a plan share a branch.
+    // Instances that batch_apart names, if their y/x passes differ, follow
+    // instead in groups of one (n1, n2): branches within a group, the groups in turn.
     vloc_plan owner = plans[0];
     const int K = std::min(ninst, (int)kBatchBranches);
     cudaError_t e;
@@ -1496,18 +1511,47 @@ int vloc_apply_batched(int ninst, const vloc_plan* plans, const void* const* c, 
     auto branched = [&](cudaStream_t cs) {
         cudaError_t er;
         if ((er = cudaEventRecord(owner->fork_event, cs))) return cuda_fail(er, "fork");
-        std::vector<int> branch_of(ninst);
+        // group of each instance: 0 together, 1.. in turn
+        std::vector<int> group(ninst, 0), branch_of(ninst, 0);
+        std::vector<std::pair<int, int>> kinds;
         for (int i = 0; i < ninst; ++i) {
-            branch_of[i] = i % K;
-            for (int j = 0; j < i; ++j)
-                if (plans[j] == plans[i]) { branch_of[i] = branch_of[j]; break; }
+            for (int j = 0; j < ninst && !group[i]; ++j) {
+                if (plans[j] != plans[i] || !batch_apart(plans[j], nb[j])) continue;
+                const std::pair<int, int> k(plans[i]->n1, plans[i]->n2);
+                group[i] = (int)(std::find(kinds.begin(), kinds.end(), k) - kinds.begin()) + 1;
+                if (group[i] > (int)kinds.size()) kinds.push_back(k);
+            }
+        }
+        if (kinds.size() < 2) {
+            std::fill(group.begin(), group.end(), 0);
+            kinds.clear();
         }
         for (int b = 0; b < K; ++b)
             if ((er = cudaStreamWaitEvent(owner->branch_streams[b], owner->fork_event, 0))) return cuda_fail(er, "fork wait");
-        for (int i = 0; i < ninst; ++i) {
-            if (nb[i] == 0) continue;
-            int rc = apply_any(plans[i], c[i], V[i], nb[i], out[i], owner->branch_streams[branch_of[i]]);
-            if (rc) return rc;
+        for (int gr = 0; gr <= (int)kinds.size(); ++gr) {
+            int members = 0;
+            for (int i = 0; i < ninst; ++i) {
+                if (group[i] != gr) continue;
+                branch_of[i] = members++ % K;
+                for (int j = 0; j < i; ++j)
+                    if (plans[j] == plans[i]) { branch_of[i] = branch_of[j]; break; }
+            }
+            // a group of several leaves branch 0 and comes back to it
+            const bool fork = gr > 0 && members > 1;
+            if (fork) {
+                if ((er = cudaEventRecord(owner->branch_events[0], owner->branch_streams[0]))) return cuda_fail(er, "group");
+                for (int b = 1; b < K; ++b)
+                    if ((er = cudaStreamWaitEvent(owner->branch_streams[b], owner->branch_events[0], 0))) return cuda_fail(er, "group wait");
+            }
+            for (int i = 0; i < ninst; ++i) {
+                if (group[i] != gr || nb[i] == 0) continue;
+                int rc = apply_any(plans[i], c[i], V[i], nb[i], out[i], owner->branch_streams[branch_of[i]]);
+                if (rc) return rc;
+            }
+            for (int b = 1; fork && b < K; ++b) {
+                if ((er = cudaEventRecord(owner->branch_events[b], owner->branch_streams[b]))) return cuda_fail(er, "group join");
+                if ((er = cudaStreamWaitEvent(owner->branch_streams[0], owner->branch_events[b], 0))) return cuda_fail(er, "group join wait");
+            }
         }
         for (int b = 0; b < K; ++b) {
             if ((er = cudaEventRecord(owner->branch_events[b], owner->branch_streams[b]))) return cuda_fail(er, "join");

@@ -156,3 +156,32 @@ def test_line_density(n, R, nb, chunk, gamma, monkeypatch):
     assert err(rho, want) < TOL["f32"]
     assert err(rho, rho0.cpu().numpy().astype(np.float64)) < 3e-7
     assert err(ones, f(n, g, c.astype(np.complex128), np.ones(nb))) < TOL["f32"]
+
+
+@pytest.mark.parametrize("spec", [
+    [(48, 8), (96, 50), (100, 41), (96, 44), (24, 5)],   # 96 twice: a group of two, then 100; the small ones beside them
+    [(96, 50), (96, 47)],                                # one kind only: together
+    [(90, 60), (108, 40), (120, 0), (90, 3)],            # no bands, and a small instance of a large length
+])
+def test_batched_groups_bit_identical(spec):
+    """Instances of a captured batch that run in turn, in groups and together
+    give what single calls give, captured and replayed, also where one plan
+    holds two of them."""
+    parts = []
+    for i, (n, nb) in enumerate(spec):
+        g = synth.sphere_glist(n, n, n, n / 4)
+        V = torch.from_numpy(synth.potential(n, n, n, "smooth", 70 + i)[0].astype(np.float32)).cuda()
+        c = torch.from_numpy(synth.coefficients(g, max(nb, 1), seed=80 + i, dtype=np.complex64)[:nb].copy()).cuda()
+        parts.append((vloc.VlocPlan((n,) * 3, g, torch.complex64, graph=True), c, V))
+    n, nb = spec[0]
+    parts.append((parts[0][0], parts[0][1][: max(1, nb // 2)].contiguous(), parts[0][2]))  # the first plan again
+    plans, cs, Vs = zip(*parts)
+    ref = [vloc.VlocPlan(p.grid, p.glist, torch.complex64).apply(c, V) for p, c, V in parts]
+    outs = [torch.empty_like(c) for c in cs]
+    for _ in range(2):
+        for o in outs:
+            o.fill_(float("nan"))
+        vloc.apply_batched(plans, cs, Vs, outs)
+        torch.cuda.synchronize()
+        for o, r in zip(outs, ref):
+            assert torch.equal(o, r)
