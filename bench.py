@@ -35,8 +35,8 @@ FALLBACK_HBM_GBS = 6800.0
 # the two arms share this config dict (the workload); arm details go elsewhere
 CONFIG = {"workload": WORKLOAD, "grid": list(GRID), "npw": 57777, "bands_per_gpu": NBANDS,
           "l2": "inputs larger than L2 (473 MB in + 473 MB out per step)", "parallelism": "bands split over GPUs"}
-KERNEL_SOURCES = ["paper_1601_07378_gb300/csrc/fft_core.cuh", "paper_1601_07378_gb300/csrc/fft_ct.cuh",
-                  "paper_1601_07378_gb300/csrc/kernels_impl.cuh", "paper_1601_07378_gb300/csrc/kernels_ct.cuh"]
+KERNEL_SOURCES = ["paper_1601_07378_gb300/csrc/fft_core.cuh", "paper_1601_07378_gb300/csrc/line_dft.cuh",
+                  "paper_1601_07378_gb300/csrc/kernels_line.h", "paper_1601_07378_gb300/csrc/kernels_line.cuh"]
 
 
 def env_int(name, default):
@@ -72,6 +72,21 @@ def path_counts(info, n):
     B5 = 2 * npw * e + 4 * cyl * e + 4 * slab * e
     B3 = 2 * npw * e + 4 * slab * e
     return per_band, flops, B5, B3
+
+
+def fused_counts(info, n):
+    """The same for the three-launch form (z-pass, fused y/x pass, z-pass; V
+    transposed once a call): the kernels move the sticks, never the slab.
+    Returns bytes per band by profile slot, their sum, and the fused pass's
+    share of the flops."""
+    n1, n2, n3 = n
+    e = 8 if info["precision"] == 1 else 16
+    cyl = info["nsticks"] * n3
+    per_band = {"k1_scatter_zpass": (info["npw"] + cyl) * e, "k3_xpass_v": 2 * cyl * e,
+                "k4_zpass_gather": (cyl + info["npw"]) * e}
+    f = lambda m: 5.0 * m * math.log2(m)
+    yx_flops = 2 * (info["nplanes"] * n3 * f(n2) + n2 * n3 * f(n1)) + 2 * n1 * n2 * n3
+    return per_band, sum(per_band.values()), yx_flops
 
 
 def kernel_src_sha() -> str:
@@ -375,7 +390,14 @@ def run_ours(args, rank, world, local_rank):
     dom = max(prof, key=lambda k: prof[k][1])
     nl, tms = prof[dom]
     bands_per_launch = NBANDS * args.steps / nl
-    bytes_launch = per_band[dom] * bands_per_launch + (GRID[0] * GRID[1] * GRID[2] * 4 if dom == "k3_xpass_v" else 0)
+    # three launches (no y-pass slot) or the five-launch chain: the bytes of
+    # each kernel differ
+    fused = "k2_ypass_inv" not in prof
+    fused_band, moved, yx_flops = fused_counts(info, GRID)
+    if not fused:
+        moved = B5
+    bytes_launch = (fused_band if fused else per_band)[dom] * bands_per_launch + \
+        (GRID[0] * GRID[1] * GRID[2] * 4 if dom == "k3_xpass_v" else 0)
     achieved = bytes_launch / (tms / nl / 1e3) / 1e9
     peak, peak_kind = peaks()
     tr = load_traffic(dom, "f32")
@@ -384,10 +406,15 @@ def run_ours(args, rank, world, local_rank):
                 "traffic": tr * bands_per_launch if tr is not None else None,
                 "alg_bytes_per_launch": bytes_launch, "bands_per_launch": bands_per_launch,
                 "kernel_share": {k: round(v[1] / tot, 4) for k, v in prof.items()}}
-    path = {"B5_bytes_per_band": B5, "B3_bytes_per_band": B3,
+    yx_gflops = yx_flops * bands_per_launch / (tms / nl / 1e3) / 1e9 if fused and dom == "k3_xpass_v" else None
+    path = {"launch_form": "z, fused y/x, z" if fused else "five launches", "moved_bytes_per_band": moved,
+            "frac_of_moved_bytes_roofline": value / world / (peak * 1e9 / moved),
+            "B5_bytes_per_band": B5, "B3_bytes_per_band": B3,
             "frac_of_B5_roofline": value / world / (peak * 1e9 / B5),
             "frac_of_B3_roofline": value / world / (peak * 1e9 / B3),
-            "flops_per_band": flops, "gflops": value / world * flops / 1e9}
+            "flops_per_band": flops, "gflops": value / world * flops / 1e9,
+            "what": "B5/B3: bytes of the five-launch and the plane-fused chain; the fused form moves "
+                    "moved_bytes_per_band and its y/x pass is bound by FP32 issue (roofline.bound = alu)"}
 
     # ---- adjoint FP32
     ms_adj = time_steps(lambda: plan.apply(c_d, V_d, out=out_d, adjoint=True), args.steps, 2, stream, dist_on)
@@ -448,6 +475,14 @@ def run_ours(args, rank, world, local_rank):
 
     # ---- measured arithmetic ceilings (FP64 and FP32 pipes) for the FP64 legs
     alu = measure_alu_peaks(local_rank)
+
+    if yx_gflops is not None:
+        # the fused pass moves too few bytes to be bound by HBM: its roofline
+        # is the measured FP32 rate; the HBM figures stay beside it
+        roofline.update({"bound": "alu", "achieved": yx_gflops, "peak": alu["ffma2_gflops"], "unit": "GFLOP/s",
+                         "frac": yx_gflops / alu["ffma2_gflops"],
+                         "peak_source": "measured (vloc_alu_peak paired FFMA, this run); achieved in 5 N log2 N",
+                         "hbm_achieved_GBps": achieved, "hbm_peak_GBps": peak, "hbm_frac": achieved / peak})
 
     # ---- FP64 path
     plan64 = vloc.VlocPlan(GRID, g, torch.complex128)
@@ -526,17 +561,21 @@ def run_ours(args, rank, world, local_rank):
         grid_d = torch.empty((nh, *GRID), dtype=torch.complex64, device="cuda")
         rho_d = torch.empty(GRID, dtype=torch.float32, device="cuda")
         kh = max(3, args.steps // 2)
+        plan.profile(True)
+        plan.density(c_d, rho=rho_d)
+        dens_fused = "k2_ypass_inv" not in plan.get_profile()
+        plan.profile(False)
         halves = {
             "to_real": leg(lambda: plan.to_real(c_d[:nh], grid_d), kh, nh,
                            info["npw"] * 8 + 2 * cyl_b + 2 * slab_b + Nn * 8),
             "to_recip": leg(lambda: plan.to_recip(grid_d, out_d[:nh]), kh, nh,
                             Nn * 8 + 2 * slab_b + 2 * cyl_b + info["npw"] * 8),
             "density": leg(lambda: plan.density(c_d, rho=rho_d), kh, NBANDS,
-                           info["npw"] * 8 + 2 * cyl_b + 2 * slab_b),
+                           info["npw"] * 8 + 2 * cyl_b + (0 if dens_fused else 2 * slab_b)),
             "what": "96^3, R = 24, FP32: psi = F+ S c to full grids (256 bands), r -> G of full grids "
                     "(256 bands), rho = sum |psi_n|^2 (1024 bands); alg bytes per band, every "
                     "inter-kernel round trip counted as in B5: to_real/to_recip npw + 2 cyl + 2 slab + N, "
-                    "density npw + 2 cyl + 2 slab (complex64)",
+                    "density npw + 2 cyl (+ 2 slab in the five-launch form) (complex64)",
         }
         del grid_d, rho_d
 
@@ -602,8 +641,9 @@ def run_ours(args, rank, world, local_rank):
                    "serial_direct_ms_per_step": mss / kb,
                    "serial_direct_frac_of_hbm": alg / (mss / kb / 1e3) / (peak * 1e9),
                    "what": "8 instances 48^3..144^3, R = n/4, 64..512 bands, FP32, one CUDA graph "
-                           "(instances on up to 4 parallel branches); serial_direct: the same plans' "
-                           "applies one after another without a graph; bytes: sum of B5 x bands"}
+                           "(large instances of different lengths in turn, the rest on up to 4 parallel branches); serial_direct: the same plans' "
+                           "applies one after another without a graph; bytes: sum of B5 x bands, the "
+                           "five-launch chain's (instances in the fused form move fewer)"}
         del insts, bplans, bcs, bVs, bouts, splans
 
     # ---- differentiable apply: loss = sum_n <psi_n|V|psi_n> + ||V psi - t||^2,
