@@ -280,8 +280,8 @@ int vloc_density(vloc_plan plan, const void* coeffs, const void* occ, int64_t nb
  * and spheres).  Without VLOC_GRAPH they are enqueued back to back on the
  * stream.  When every plan has VLOC_GRAPH the whole batch is captured once
  * (per pointer set) into one CUDA graph whose instances run as up to four
- * parallel branches (instances sharing a plan share a branch), and each
- * call is one graph launch.  Arrays have ninst entries each; plans must
+ * parallel branches (instances sharing a plan share a branch; large ones of
+ * different lengths follow one another), and each call is one graph launch.  Arrays have ninst entries each; plans must
  * share a precision.  Errors as vloc_apply, per instance.
  */
 int vloc_apply_batched(int ninst, const vloc_plan* plans, const void* const* coeffs,
