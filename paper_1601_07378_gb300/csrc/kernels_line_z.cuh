@@ -50,10 +50,12 @@ template <bool GM> __device__ __forceinline__ bool dense_rows(const Tables& t, i
 // inverse's first, the forward's last).  ED (caller lists in stick order): a warp
 // takes 8 line pairs and 4 consecutive units instead of 16 and 2, so that an
 // access covers 32 bytes of each stick's run; these accesses are most of a
-// block's load/store wavefronts.  96^3 x 1024 bands: inverse 0.452 -> 0.449 ms,
-// forward 0.432 -> 0.424; 128^3 x 256: 0.263 -> 0.263, 0.267 -> 0.261.  Lists in
-// another order have no runs to cover and lose rows of the table that two units
-// share (shuffled, 96^3: 0.653 -> 0.673, 0.516 -> 0.524), so they keep 16 and 2.
+// block's load/store wavefronts.  Forward 0.430 -> 0.422 ms (96^3 x 1024 bands),
+// 0.266 -> 0.259 (128^3 x 256); inverse 0.266 -> 0.259 (120^3 x 256), 0.0875 ->
+// 0.0861 (64^3 x 512), 96^3 x 1024 0.452 -> 0.449 on one GPU and 0.470 -> 0.473
+// on another.  Lists in another order have no runs to cover and lose rows of the
+// table that two units share (shuffled, 96^3: 0.653 -> 0.673, 0.516 -> 0.524),
+// so they keep 16 and 2.
 template <bool ED> __device__ __forceinline__ int edge_slot() {
     return ED ? (threadIdx.x & 7) + ((threadIdx.x >> 5) & 1) * 8 : slot_of();
 }
@@ -196,23 +198,31 @@ __global__ void __launch_bounds__(kThreads, GM ? minb_k4q(N, true) : minb_k4d(N)
     SmemP sb{buf};
     RevStage<N, -1, W, 0>::template run<false>(stw, dr, sb, slot, sub, warp, act);
     load_tw<float>(stw, tw3, N);
-    __syncthreads();
     if constexpr (!GM) {
-        if (!ED && !act) return;  // ED: `act` is not this lane's line pair; the table's -1 drops absent ones
+        // The table's entries are requested before the barrier where a thread
+        // has one unit (64^3 x 512 bands 0.078 -> 0.071 ms, 96^3 x 1024 0.422 ->
+        // 0.422, shuffled list 0.512 -> 0.510); with two they cost registers
+        // (120^3 x 256 0.2234 -> 0.2243).
+        constexpr bool AHEAD = L::U == 1;
         const int slot = edge_slot<ED>();
         const int* zd = t.zd + (size_t)g * (QR::groups() * NA) * 32 + 2 * slot;
+        int2 e[R0];
+        auto entries = [&](int i) {
+            sfor<R0>([&](auto rc) {
+                constexpr int r = decltype(rc)::value;
+                if constexpr (QR::kind(r) != 0) e[r] = *reinterpret_cast<const int2*>(zd + (QR::group(r) * NA + i) * 32);
+            });
+        };
+        if (AHEAD && (L::NI % (2 * W) == 0 || edge_unit<ED>() < L::NI)) entries(edge_unit<ED>());
+        __syncthreads();
+        if (!ED && !act) return;  // ED: `act` is not this lane's line pair; the table's -1 drops absent ones
         float2* o = out + b * t.npw;
         const float2* ci = diag ? cin + b * t.npw : cin;
 #pragma unroll
         for (int u = 0; u < L::U; ++u) {
             const int i = edge_unit<ED>() + 2 * W * u;
             if (L::NI % (2 * W) == 0 || i < L::NI) {
-                int2 e[R0];
-                sfor<R0>([&](auto rc) {
-                    constexpr int r = decltype(rc)::value;
-                    if constexpr (QR::kind(r) != 0)
-                        e[r] = *reinterpret_cast<const int2*>(zd + (QR::group(r) * NA + i) * 32);
-                });
+                if (!AHEAD) entries(i);
                 P2f h[R0];
                 L::compute_unit(h, stw, sb, i, slot);
                 sfor<R0>([&](auto rc) {
@@ -235,6 +245,7 @@ __global__ void __launch_bounds__(kThreads, GM ? minb_k4q(N, true) : minb_k4d(N)
             }
         }
     } else {
+        __syncthreads();
         P2f h[L::U][R0];
         if (act) L::compute(h, stw, sb, slot, sub, warp);
         __syncthreads();
