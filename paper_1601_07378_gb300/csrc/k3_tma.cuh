@@ -190,9 +190,7 @@ __global__ void __launch_bounds__(kThreads, 4) k3_tma(DevTables t, const float2*
 template <int N>
 int launch_k3_tma(const DevTables& t, const void* tw1, const void* V, long long nb, void* slab, const K3Tma& tma,
                   cudaStream_t st) {
-    static const cudaError_t once =
-        cudaFuncSetAttribute(k3_tma<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k3_tma_smem(N, N));
-    if (once) return (int)once;
+    if (const cudaError_t e = smem_optin<k3_tma<N>>(k3_tma_smem(N, N))) return (int)e;
     static int nsm = 0;
     if (!nsm) {
         int dev = 0;

@@ -1521,10 +1521,6 @@ __global__ void __launch_bounds__(kThreads, N <= 96 ? VLOC_MINB_K3DQ : 1) k3dq_c
 // ------------------------------------------------------------ launchers
 template <int N> struct CtSmem {
     static constexpr size_t sm = ct_smem<N>();
-    template <class K> static cudaError_t ensure(K kernel) {
-        if (sm <= 48 * 1024) return cudaSuccess;
-        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    }
 };
 
 // K1 over nb bands (GM: nb Gamma-point pairs formed from the caller's real
@@ -1542,9 +1538,7 @@ int launch_k1_ct(const DevTables& t, const void* tw3, const void* coeffs, long l
     if constexpr (Sched<N>::nst == 2) {
         if (!GM && VLOC_K1_BULK && t.runs == 1 && t.zd_rows == QRows<N>::groups() * QRows<N>::NA) {
             constexpr size_t sm = k1b_smem<N>();
-            static const cudaError_t onceb =
-                sm <= 48 * 1024 ? cudaSuccess : cudaFuncSetAttribute(k1b_ct<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-            if (onceb) return (int)onceb;
+            if (const cudaError_t e = smem_optin<k1b_ct<N>>(sm)) return (int)e;
             k1b_ct<N><<<dim3(t.T, (unsigned)nb), kThreads, sm, st>>>(t, (const float2*)tw3, (const float2*)coeffs,
                                                                     (float2*)cyl);
             return (int)cudaGetLastError();
@@ -1553,25 +1547,21 @@ int launch_k1_ct(const DevTables& t, const void* tw3, const void* coeffs, long l
         // indices of the complex band the kernel reads)
         if (!GM && VLOC_K1_DIRECT && t.zd_rows == QRows<N>::groups() * QRows<N>::NA) {
             if (t.runs == 2) {
-                static const cudaError_t oncer = CtSmem<N>::ensure(k1d_ct<N, true>);
-                if (oncer) return (int)oncer;
+                if (const cudaError_t e = smem_optin<k1d_ct<N, true>>(CtSmem<N>::sm)) return (int)e;
                 return pdl_launch(k1d_ct<N, true>, dim3(t.T, (unsigned)nb), kThreads, CtSmem<N>::sm, st, t, (const
                     float2*)tw3, (const float2*)coeffs, (float2*)cyl);
             }
-            static const cudaError_t onced = CtSmem<N>::ensure(k1d_ct<N, false>);
-            if (onced) return (int)onced;
+            if (const cudaError_t e = smem_optin<k1d_ct<N, false>>(CtSmem<N>::sm)) return (int)e;
             return pdl_launch(k1d_ct<N, false>, dim3(t.T, (unsigned)nb), kThreads, CtSmem<N>::sm, st, t, (const
                 float2*)tw3, (const float2*)coeffs, (float2*)cyl);
         }
         if (t.zq) {
-            static const cudaError_t onceq = CtSmem<N>::ensure(k1q_ct<N, GM>);
-            if (onceq) return (int)onceq;
+            if (const cudaError_t e = smem_optin<k1q_ct<N, GM>>(CtSmem<N>::sm)) return (int)e;
             return pdl_launch(k1q_ct<N, GM>, dim3(t.T, (unsigned)nb), kThreads, CtSmem<N>::sm, st, t, (const
                 float2*)tw3, (const float2*)coeffs, (float2*)cyl, g);
         }
     }
-    static const cudaError_t once = CtSmem<N>::ensure(k1_ct<N, GM>);
-    if (once) return (int)once;
+    if (const cudaError_t e = smem_optin<k1_ct<N, GM>>(CtSmem<N>::sm)) return (int)e;
     return pdl_launch(k1_ct<N, GM>, dim3(t.T, (unsigned)nb), kThreads, CtSmem<N>::sm, st, t, (const float2*)tw3,
         (const float2*)coeffs, (float2*)cyl, g);
 }
@@ -1591,13 +1581,11 @@ int LaunchCT<T, N>::k2(int sign, const DevTables& t, const void* tw2, long long 
                        cudaStream_t st) {
     const dim3 grid(t.NP, (t.n3 + kLines - 1) / kLines, (unsigned)nb);
     if (sign > 0) {
-        static const cudaError_t once = CtSmem<N>::ensure(k2_ct<+1, N>);
-        if (once) return (int)once;
+        if (const cudaError_t e = smem_optin<k2_ct<+1, N>>(CtSmem<N>::sm)) return (int)e;
         return pdl_launch(k2_ct<+1, N>, grid, kThreads, CtSmem<N>::sm, st, t, (const float2*)tw2, (float2*)cyl,
             (float2*)slab);
     } else {
-        static const cudaError_t once = CtSmem<N>::ensure(k2_ct<-1, N>);
-        if (once) return (int)once;
+        if (const cudaError_t e = smem_optin<k2_ct<-1, N>>(CtSmem<N>::sm)) return (int)e;
         return pdl_launch(k2_ct<-1, N>, grid, kThreads, CtSmem<N>::sm, st, t, (const float2*)tw2, (float2*)cyl,
             (float2*)slab);
     }
@@ -1627,8 +1615,7 @@ int LaunchCT<T, N>::k3(const DevTables& t, const void* tw1, const void* V, long 
             }
         }
     }
-    static const cudaError_t once = CtSmem<N>::ensure(k3_ct<N, W>);
-    if (once) return (int)once;
+    if (const cudaError_t e = smem_optin<k3_ct<N, W>>(CtSmem<N>::sm)) return (int)e;
     const dim3 grid(t.n2, (t.n3 + kLines - 1) / kLines, (unsigned)nb);
     return pdl_launch(k3_ct<N, W>, grid, 32 * W, CtSmem<N>::sm, st, t, (const float2*)tw1, (const float*)V,
         (float2*)slab);
@@ -1637,18 +1624,13 @@ template <typename T, int N>
 int LaunchCT<T, N>::k3b(const DevTables& t, const void* tw1, const void* sc, const void* sg, long long nb, int bpg,
                         double* partial, cudaStream_t st) {
     constexpr size_t sm = 2 * (size_t)N * kLdP * sizeof(float2) + (size_t)N * sizeof(float2) + (size_t)N * sizeof(int) + 16;
-    static const cudaError_t once =
-        sm <= 48 * 1024 ? cudaSuccess : cudaFuncSetAttribute(k3b_ct<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (once) return (int)once;
+    if (const cudaError_t e = smem_optin<k3b_ct<N>>(sm)) return (int)e;
     const int ng = (int)((nb + bpg - 1) / bpg);
     const dim3 grid(t.n2, (t.n3 + kLines - 1) / kLines, ng);
     const double invN = 1.0 / ((double)t.n1 * t.n2 * t.n3);
     if constexpr (Sched<N>::nst == 2) {
         if (t.xq) {
-            static const cudaError_t onceq =
-                sm <= 48 * 1024 ? cudaSuccess
-                                : cudaFuncSetAttribute(k3bq_ct<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-            if (onceq) return (int)onceq;
+            if (const cudaError_t e = smem_optin<k3bq_ct<N>>(sm)) return (int)e;
             k3bq_ct<N><<<grid, kThreads, sm, st>>>(t, (const float2*)tw1, (const float2*)sc, (const float2*)sg, (int)nb,
                                                   bpg, partial, invN);
             return (int)cudaGetLastError();
@@ -1663,12 +1645,10 @@ int LaunchCT<T, N>::k3g(int sign, const DevTables& t, const void* tw1, long long
                         cudaStream_t st) {
     const dim3 g3(t.n2, (t.n3 + kLines - 1) / kLines, (unsigned)nb);
     if (sign > 0) {
-        static const cudaError_t once = CtSmem<N>::ensure(k3g_ct<+1, N>);
-        if (once) return (int)once;
+        if (const cudaError_t e = smem_optin<k3g_ct<+1, N>>(CtSmem<N>::sm)) return (int)e;
         k3g_ct<+1, N><<<g3, kThreads, CtSmem<N>::sm, st>>>(t, (const float2*)tw1, (float2*)slab, (float2*)grid);
     } else {
-        static const cudaError_t once = CtSmem<N>::ensure(k3g_ct<-1, N>);
-        if (once) return (int)once;
+        if (const cudaError_t e = smem_optin<k3g_ct<-1, N>>(CtSmem<N>::sm)) return (int)e;
         k3g_ct<-1, N><<<g3, kThreads, CtSmem<N>::sm, st>>>(t, (const float2*)tw1, (float2*)slab, (float2*)grid);
     }
     return (int)cudaGetLastError();
@@ -1680,15 +1660,13 @@ int LaunchCT<T, N>::k3d(const DevTables& t, const void* tw1, const void* slab, l
     const dim3 grid(t.n2, (t.n3 + kLines - 1) / kLines, ng);
     if constexpr (Sched<N>::nst == 2) {
         if (t.xq) {
-            static const cudaError_t onceq = CtSmem<N>::ensure(k3dq_ct<N>);
-            if (onceq) return (int)onceq;
+            if (const cudaError_t e = smem_optin<k3dq_ct<N>>(CtSmem<N>::sm)) return (int)e;
             k3dq_ct<N><<<grid, kThreads, CtSmem<N>::sm, st>>>(t, (const float2*)tw1, (const float2*)slab, (int)nb, bpg,
                                                               (const float*)occ, b_base, pair, nreal, partial);
             return (int)cudaGetLastError();
         }
     }
-    static const cudaError_t once = CtSmem<N>::ensure(k3d_ct<N>);
-    if (once) return (int)once;
+    if (const cudaError_t e = smem_optin<k3d_ct<N>>(CtSmem<N>::sm)) return (int)e;
     k3d_ct<N><<<grid, kThreads, CtSmem<N>::sm, st>>>(t, (const float2*)tw1, (const float2*)slab, (int)nb, bpg,
                                                      (const float*)occ, b_base, pair, nreal, partial);
     return (int)cudaGetLastError();
@@ -1706,20 +1684,17 @@ int launch_k4_ct(const DevTables& t, const void* tw3, const void* cyl, long long
     }
     if constexpr (Sched<N>::nst == 2) {
         if (!GM && VLOC_K4_DIRECT && t.zd_rows == QRows<N>::groups() * QRows<N>::NA) {
-            static const cudaError_t onced = CtSmem<N>::ensure(k4d_ct<N>);
-            if (onced) return (int)onced;
+            if (const cudaError_t e = smem_optin<k4d_ct<N>>(CtSmem<N>::sm)) return (int)e;
             return pdl_launch(k4d_ct<N>, dim3(t.T, (unsigned)nb), kThreads, CtSmem<N>::sm, st, t, (const float2*)tw3,
                 (const float2*)cyl, (float2*)out, scale, (const float*)diag, (const float2*)cin);
         }
         if (t.zq) {
-            static const cudaError_t onceq = CtSmem<N>::ensure(k4q_ct<N, GM>);
-            if (onceq) return (int)onceq;
+            if (const cudaError_t e = smem_optin<k4q_ct<N, GM>>(CtSmem<N>::sm)) return (int)e;
             return pdl_launch(k4q_ct<N, GM>, dim3(t.T, (unsigned)nb), kThreads, CtSmem<N>::sm, st, t, (const
                 float2*)tw3, (const float2*)cyl, (float2*)out, scale, (const float*)diag, (const float2*)cin, g);
         }
     }
-    static const cudaError_t once = CtSmem<N>::ensure(k4_ct<N, GM>);
-    if (once) return (int)once;
+    if (const cudaError_t e = smem_optin<k4_ct<N, GM>>(CtSmem<N>::sm)) return (int)e;
     return pdl_launch(k4_ct<N, GM>, dim3(t.T, (unsigned)nb), kThreads, CtSmem<N>::sm, st, t, (const float2*)tw3,
         (const float2*)cyl, (float2*)out, scale, (const float*)diag, (const float2*)cin, g);
 }

@@ -617,10 +617,6 @@ __global__ void __launch_bounds__(kThreads, MINB) k4_wb(DevTables t, const typen
 // ------------------------------------------------------------ launchers
 template <class Pol, int N> struct WSmem {
     static constexpr size_t sm = w_smem<Pol, N>();
-    template <class K> static cudaError_t ensure(K kernel) {
-        if (sm <= 48 * 1024) return cudaSuccess;
-        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    }
 };
 
 template <int P, int N>
@@ -630,26 +626,22 @@ int LaunchF64<P, N>::k1(const DevTables& t, const void* tw3, const void* coeffs,
     if constexpr (Sched<N>::nst == 2) {
         if (VLOC_DF_DIRECT_Z && t.zd_rows == QRows<N>::groups() * QRows<N>::NA) {
             if constexpr (df_floors<Pol, N>()) {
-                static const cudaError_t onced = WSmem<Pol, N>::ensure(k1d_wb<Pol, N, VLOC_MINB_K1DF>);
-                if (onced) return (int)onced;
+                if (const cudaError_t e = smem_optin<k1d_wb<Pol, N, VLOC_MINB_K1DF>>(WSmem<Pol, N>::sm)) return (int)e;
                 return pdl_launch(k1d_wb<Pol, N, VLOC_MINB_K1DF>, dim3(t.T, (unsigned)nb, 2), kThreads, WSmem<Pol,
                     N>::sm, st, t, (const typename Pol::TW*)tw3, (const double2*)coeffs, (typename Pol::V*)cyl);
             } else {
-                static const cudaError_t onced = WSmem<Pol, N>::ensure(k1d_w<Pol, N>);
-                if (onced) return (int)onced;
+                if (const cudaError_t e = smem_optin<k1d_w<Pol, N>>(WSmem<Pol, N>::sm)) return (int)e;
                 return pdl_launch(k1d_w<Pol, N>, dim3(t.T, (unsigned)nb, 2), kThreads, WSmem<Pol, N>::sm, st, t,
                     (const typename Pol::TW*)tw3, (const double2*)coeffs, (typename Pol::V*)cyl);
             }
         }
     }
     if constexpr (df_floors<Pol, N>()) {
-        static const cudaError_t onceb = WSmem<Pol, N>::ensure(k1_wb<Pol, N, VLOC_MINB_K1DF>);
-        if (onceb) return (int)onceb;
+        if (const cudaError_t e = smem_optin<k1_wb<Pol, N, VLOC_MINB_K1DF>>(WSmem<Pol, N>::sm)) return (int)e;
         return pdl_launch(k1_wb<Pol, N, VLOC_MINB_K1DF>, dim3(t.T, (unsigned)nb, 2), kThreads, WSmem<Pol, N>::sm, st,
             t, (const typename Pol::TW*)tw3, (const double2*)coeffs, (typename Pol::V*)cyl);
     } else {
-        static const cudaError_t once = WSmem<Pol, N>::ensure(k1_w<Pol, N>);
-        if (once) return (int)once;
+        if (const cudaError_t e = smem_optin<k1_w<Pol, N>>(WSmem<Pol, N>::sm)) return (int)e;
         return pdl_launch(k1_w<Pol, N>, dim3(t.T, (unsigned)nb, 2), kThreads, WSmem<Pol, N>::sm, st, t, (const
             typename Pol::TW*)tw3, (const double2*)coeffs, (typename Pol::V*)cyl);
     }
@@ -660,12 +652,10 @@ int launch_k2w(const DevTables& t, const typename Pol::TW* tw2, long long nb, ty
     const dim3 grid(t.NP, (t.n3 + kLinesDF - 1) / kLinesDF, (unsigned)nb);
     if constexpr (df_floors<Pol, N>()) {
         constexpr int MINB = S > 0 ? VLOC_MINB_K2IDF : VLOC_MINB_K2FDF;
-        static const cudaError_t onceb = WSmem<Pol, N>::ensure(k2_wb<Pol, S, N, Q, MINB>);
-        if (onceb) return (int)onceb;
+        if (const cudaError_t e = smem_optin<k2_wb<Pol, S, N, Q, MINB>>(WSmem<Pol, N>::sm)) return (int)e;
         return pdl_launch(k2_wb<Pol, S, N, Q, MINB>, grid, kThreads, WSmem<Pol, N>::sm, st, t, tw2, cyl, slab);
     } else {
-        static const cudaError_t once = WSmem<Pol, N>::ensure(k2_w<Pol, S, N, Q>);
-        if (once) return (int)once;
+        if (const cudaError_t e = smem_optin<k2_w<Pol, S, N, Q>>(WSmem<Pol, N>::sm)) return (int)e;
         return pdl_launch(k2_w<Pol, S, N, Q>, grid, kThreads, WSmem<Pol, N>::sm, st, t, tw2, cyl, slab);
     }
 }
@@ -689,16 +679,12 @@ int LaunchF64<P, N>::k3(const DevTables& t, const void* tw1, const void* V, long
     if constexpr (Sched<N>::nst == 2) {
         if (t.xq) {
             constexpr size_t sm = k3q_w_smem<Pol, N>();
-            static const cudaError_t onceq =
-                sm <= 48 * 1024 ? cudaSuccess
-                                : cudaFuncSetAttribute(k3q_w<Pol, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-            if (onceq) return (int)onceq;
+            if (const cudaError_t e = smem_optin<k3q_w<Pol, N>>(sm)) return (int)e;
             return pdl_launch(k3q_w<Pol, N>, grid, kThreads, sm, st, t, (const typename Pol::TW*)tw1, (const typename
                 Pol::VR*)V, (typename Pol::V*)slab);
         }
     }
-    static const cudaError_t once = WSmem<Pol, N>::ensure(k3_w<Pol, N>);
-    if (once) return (int)once;
+    if (const cudaError_t e = smem_optin<k3_w<Pol, N>>(WSmem<Pol, N>::sm)) return (int)e;
     return pdl_launch(k3_w<Pol, N>, grid, kThreads, WSmem<Pol, N>::sm, st, t, (const typename Pol::TW*)tw1, (const
         typename Pol::VR*)V, (typename Pol::V*)slab);
 }
@@ -708,13 +694,11 @@ int launch_k4w(const DevTables& t, const typename Pol::TW* tw3, const typename P
     const double scale = 1.0 / ((double)t.n1 * t.n2 * t.n3);
     const dim3 grid(t.T, (unsigned)nb, 2);
     if constexpr (df_floors<Pol, N>()) {
-        static const cudaError_t onceb = WSmem<Pol, N>::ensure(k4_wb<Pol, N, Q, VLOC_MINB_K4DF>);
-        if (onceb) return (int)onceb;
+        if (const cudaError_t e = smem_optin<k4_wb<Pol, N, Q, VLOC_MINB_K4DF>>(WSmem<Pol, N>::sm)) return (int)e;
         return pdl_launch(k4_wb<Pol, N, Q, VLOC_MINB_K4DF>, grid, kThreads, WSmem<Pol, N>::sm, st, t, tw3, cyl, out,
                           scale, diag, cin);
     } else {
-        static const cudaError_t once = WSmem<Pol, N>::ensure(k4_w<Pol, N, Q>);
-        if (once) return (int)once;
+        if (const cudaError_t e = smem_optin<k4_w<Pol, N, Q>>(WSmem<Pol, N>::sm)) return (int)e;
         return pdl_launch(k4_w<Pol, N, Q>, grid, kThreads, WSmem<Pol, N>::sm, st, t, tw3, cyl, out, scale, diag, cin);
     }
 }

@@ -22,6 +22,7 @@
 #include "fft_core.cuh"
 #include "internal.h"
 #include "pdl.cuh"
+#include "smem_optin.cuh"
 
 namespace vloc {
 

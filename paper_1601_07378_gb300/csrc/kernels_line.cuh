@@ -25,6 +25,7 @@
 #include "kernels_line.h"
 #include "line_dft.cuh"
 #include "pdl.cuh"
+#include "smem_optin.cuh"
 
 namespace vloc {
 namespace line {
@@ -258,15 +259,10 @@ __global__ void __launch_bounds__(64 * YX<CLS, N1, N2>::PAIRS, YX<CLS, N1, N2>::
 }
 
 // ------------------------------------------------------------ launchers
-template <class K> cudaError_t line_smem(K kernel, size_t bytes) {
-    if (bytes <= 48 * 1024) return cudaSuccess;
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
 template <int CLS, int N1, int N2>
 int launch_yx_n(const Tables& t, const float2* tw2, const float* VT, long long nb, float2* D, cudaStream_t st) {
     using C = YX<CLS, N1, N2>;
-    static const cudaError_t once = line_smem(kl_yx<CLS, N1, N2>, C::smem);
-    if (once) return (int)once;
+    if (const cudaError_t e = smem_optin<kl_yx<CLS, N1, N2>>(C::smem)) return (int)e;
     // bands per block, as measured (8 against 4: 2.28 and 2.30 ms at 96^3 x
     // 1024, 0.342 and 0.334 at 80^3 x 256, 0.956 and 0.931 at 100^3, 1.62 and
     // 1.59 at 128^3), but few enough that the grid is four waves deep

@@ -77,8 +77,7 @@ template <int CLS, int N1, int N2>
 int launch_dens_n(const Tables& t, const float2* D, long long nb, int bpg, const float* occ, long long b_base, int pair,
                   long long nreal, float* partial, cudaStream_t st) {
     using C = YXD<CLS, N1, N2>;
-    static const cudaError_t once = line_smem(kl_dens<CLS, N1, N2>, C::smem);
-    if (once) return (int)once;
+    if (const cudaError_t e = smem_optin<kl_dens<CLS, N1, N2>>(C::smem)) return (int)e;
     return pdl_launch(kl_dens<CLS, N1, N2>, dim3(t.n3, (unsigned)((nb + bpg - 1) / bpg)), 64 * C::PAIRS, C::smem, st,
         t, D, (int)nb, bpg, occ, b_base, pair, nreal, partial);
 }

@@ -273,8 +273,7 @@ __global__ void __launch_bounds__(kThreads, GM ? minb_k4q(N, true) : minb_k4d(N)
 template <int N, int MODE>
 int launch_z_inv_n(const Tables& t, const float2* tw3, const float2* c, long long nb, long long nreal, float2* D,
                    cudaStream_t st) {
-    static const cudaError_t once = CtSmem<N>::ensure(kl_z_inv<N, MODE>);
-    if (once) return (int)once;
+    if (const cudaError_t e = smem_optin<kl_z_inv<N, MODE>>(CtSmem<N>::sm)) return (int)e;
     return pdl_launch(kl_z_inv<N, MODE>, dim3(t.G, (unsigned)nb), kThreads, CtSmem<N>::sm, st, t, tw3, c, nreal, D);
 }
 template <int N>
@@ -287,8 +286,7 @@ int LaunchZ<N>::inv(const Tables& t, const float2* tw3, const float2* c, long lo
 template <int N, bool GM, bool ED>
 int launch_z_fwd_n(const Tables& t, const float2* tw3, const float2* D, long long nb, long long nreal, float2* out,
                    const float* diag, const float2* c, cudaStream_t st) {
-    static const cudaError_t once = CtSmem<N>::ensure(kl_z_fwd<N, GM, ED>);
-    if (once) return (int)once;
+    if (const cudaError_t e = smem_optin<kl_z_fwd<N, GM, ED>>(CtSmem<N>::sm)) return (int)e;
     const float scale = (float)(1.0 / ((double)t.n1 * t.n2 * t.n3));
     return pdl_launch(kl_z_fwd<N, GM, ED>, dim3(t.G, (unsigned)nb), kThreads, CtSmem<N>::sm, st, t, tw3, D, nreal, out,
         scale, diag, c);

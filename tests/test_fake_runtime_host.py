@@ -1,0 +1,89 @@
+"""Host side of the library against a stand-in for the CUDA runtime
+(fake_cudart.c): each test runs a child process with it preloaded, which calls
+the C entry points on made-up device addresses and reports what the runtime
+was asked for.  No GPU, no kernel runs."""
+import json
+import os
+import shutil
+import subprocess
+import sys
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+
+# Helpers of the children: plans and calls over made-up addresses, 16-byte
+# aligned and far from each other.
+CHILD = """
+import ctypes, json, sys
+import numpy as np
+sys.path.insert(0, %r)
+from paper_1601_07378_gb300 import synth, vloc
+lib, rt = vloc.load(), ctypes.CDLL(None)
+rt.fake_set_free.argtypes = [ctypes.c_size_t]
+rt.fake_allocated.restype = ctypes.c_size_t
+rt.fake_launch_stream.restype = ctypes.c_size_t
+def plan(n, r, flags, chunk=0):
+    g = synth.sphere_glist(*n, r)
+    if flags & vloc.VLOC_GAMMA:
+        g = synth.half_sphere(g)
+    g = np.ascontiguousarray(g, dtype=np.int32)
+    h = ctypes.c_void_p()
+    rc = lib.vloc_plan_create(ctypes.byref(h), *n, g.ctypes.data_as(ctypes.POINTER(ctypes.c_int32)), len(g), flags, chunk, None)
+    assert rc == 0, rc
+    return h
+def info(h):
+    i = vloc.VlocInfo()
+    assert lib.vloc_get_info(h, ctypes.byref(i)) == 0
+    return i
+addr = lambda k: (1 << 44) + (k << 38)
+def done(x):
+    print("RESULT " + json.dumps(x))
+""" % ROOT
+
+
+@pytest.fixture(scope="module")
+def run(tmp_path_factory):
+    from paper_1601_07378_gb300 import build
+    if not sys.platform.startswith("linux") or shutil.which("gcc") is None:
+        pytest.skip("needs gcc and LD_PRELOAD")
+    build.build()
+    so = str(tmp_path_factory.mktemp("fake") / "libfake_cudart.so")
+    subprocess.check_call(["gcc", "-shared", "-fPIC", "-O1", "-Wno-builtin-declaration-mismatch",
+                           "-I" + os.path.join(build._cuda_home(), "include"), "-o", so, os.path.join(HERE, "fake_cudart.c")])
+
+    def child(code):
+        env = dict(os.environ, LD_PRELOAD=so)
+        p = subprocess.run([sys.executable, "-c", CHILD + code], env=env, capture_output=True, text=True, timeout=300)
+        assert p.returncode == 0, p.stdout + p.stderr
+        return json.loads([ln for ln in p.stdout.splitlines() if ln.startswith("RESULT ")][-1][7:])
+    return child
+
+
+# The kernels with more than 48 KB of dynamic shared memory: the fused y/x
+# passes, the FP64 and double-float passes, the dL/dV pass.
+@pytest.mark.parametrize("n,r,flags", [((96, 96, 96), 24, "VLOC_F32"), ((144, 144, 144), 36, "VLOC_F32"),
+                                       ((96, 96, 96), 24, "VLOC_F64"), ((120, 120, 120), 30, "VLOC_F64"),
+                                       ((96, 96, 96), 24, "VLOC_F64 | vloc.VLOC_DOUBLE_FLOAT"),
+                                       ((96, 96, 100), 30, "VLOC_F64"), ((54, 54, 54), 13, "VLOC_F64")])
+def test_every_device_gets_the_shared_memory_limits(run, n, r, flags):
+    """Plans on two devices in one process: the limit is the kernel's on one
+    device, so the second device's launches need it raised again; a device's
+    second call does not."""
+    out = run(f"""
+res = []
+for dev in (0, 1, 0):
+    rt.fake_set_device(dev)
+    h = plan({n!r}, {r}, vloc.{flags}, 16)
+    before = rt.fake_limits()
+    rcs = [lib.vloc_apply(h, addr(0), addr(1), 16, addr(2), None), lib.vloc_density(h, addr(0), None, 16, addr(3), None),
+           lib.vloc_backward(h, addr(0), addr(4), addr(1), 16, addr(2), addr(3), None)]
+    mid = rt.fake_limits()
+    rcs.append(lib.vloc_apply(h, addr(0), addr(1), 16, addr(2), None))
+    res.append([rcs, mid - before, rt.fake_limits() - mid])
+done(res)
+""")
+    assert [r[0] for r in out] == [[0] * 4] * 3
+    assert out[0][1] == out[1][1]      # the second device as the first
+    assert out[2][1] == 0 and [r[2] for r in out] == [0] * 3
