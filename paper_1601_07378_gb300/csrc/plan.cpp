@@ -390,10 +390,13 @@ static void free_plan(vloc_plan p) {
     delete p;
 }
 
-int vloc_plan_create(vloc_plan* out, int n1, int n2, int n3, const int32_t* g, int64_t npw, int flags,
-                     int64_t max_bands_per_chunk, void* stream) {
-    if (!out) return VLOC_ERR_ARG;
-    *out = nullptr;
+}  // extern "C"
+
+// vloc_plan_create, with or without the line path.  *grew: the plan's workspace
+// is larger for the line path's sake (its dense rows do not shrink with the
+// sphere, the slab does).
+static int create_plan(vloc_plan* out, int n1, int n2, int n3, const int32_t* g, int64_t npw, int flags,
+                       int64_t max_bands_per_chunk, void* stream, bool line_path, bool* grew) {
     if (!g || npw <= 0) return npw == 0 ? VLOC_ERR_GLIST : VLOC_ERR_ARG;
     const int prec = flags & (VLOC_F32 | VLOC_F64);
     if (prec != VLOC_F32 && prec != VLOC_F64) return VLOC_ERR_ARG;
@@ -440,7 +443,9 @@ int vloc_plan_create(vloc_plan* out, int n1, int n2, int n3, const int32_t* g, i
     if (!p) return VLOC_ERR_ALLOC;
     auto dmalloc = [&](void** ptr, size_t bytes) -> cudaError_t {
         if (fault.alloc_at == alloc_no++) return cudaErrorMemoryAllocation;
-        return cudaMalloc(ptr, bytes);
+        const cudaError_t e = cudaMalloc(ptr, bytes);
+        if (e) cudaGetLastError();  // reported here, not by a later launch's check
+        return e;
     };
     p->poison = (flags & VLOC_POISON_WORKSPACE) != 0;
     p->n1 = n1; p->n2 = n2; p->n3 = n3; p->dbl = dbl; p->flags = flags; p->npw = npw; p->N = N;
@@ -769,7 +774,7 @@ int vloc_plan_create(vloc_plan* out, int n1, int n2, int n3, const int32_t* g, i
     // ---- tables of the line path (not among the host tables: the
     // allocation-free entry runs the five-launch chain)
     LineHost lh;
-    if (!dbl && p->fast && p->lay.zq && !(flags & (VLOC_X_TMA | VLOC_Z_WARP | VLOC_Z_BULK)) &&
+    if (line_path && !dbl && p->fast && p->lay.zq && !(flags & (VLOC_X_TMA | VLOC_Z_WARP | VLOC_Z_BULK)) &&
         std::getenv("VLOC_GAMMA_PACK") == nullptr)
         lh = build_line(n1, n2, n3, stick_x, stick_row, stick_pw_ptr, pw_user, pw_z, gamma_neg, npw_user);
     // shared-memory budget of the largest kernel tile
@@ -829,8 +834,12 @@ int vloc_plan_create(vloc_plan* out, int n1, int n2, int n3, const int32_t* g, i
         if ((e = dmalloc((void**)&p->d_vdf, (size_t)N * 8))) { free_plan(p); return cuda_fail(e, "cudaMalloc(df V)"); }
     }
 
-    // ---- workspace: cylinder [chunk][S][n3] + slab [chunk][NP][n2][n3]
-    const size_t per_band = ((size_t)S * n3 + (size_t)NP * n2 * n3) * elem;
+    // ---- workspace: cylinder [chunk][S][n3] + slab [chunk][NP][n2][n3], whose
+    // place the line path's dense bands take
+    const size_t slab_elems = (size_t)NP * n2 * n3, dense_elems = p->line_on ? line::band_elems(p->lt) : 0;
+    *grew = dense_elems > slab_elems;
+    const size_t slab_band = std::max(slab_elems, dense_elems) * elem;
+    const size_t per_band = (size_t)S * n3 * elem + slab_band;
     long long chunk = max_bands_per_chunk;
     if (chunk <= 0) {
         // Enough bands per launch that every kernel runs many waves over the
@@ -848,8 +857,6 @@ int vloc_plan_create(vloc_plan* out, int n1, int n2, int n3, const int32_t* g, i
     p->chunk = chunk;
     p->ws_bands = std::max<long long>(chunk, 2);
     p->ngroups = (int)((std::max<long long>(1, p->ws_bands / 2) + kGradBandsPerGroup - 1) / kGradBandsPerGroup);
-    // the line path's dense bands take the slab's place
-    const size_t slab_band = std::max((size_t)NP * n2 * n3 * elem, p->line_on ? line::band_elems(p->lt) * elem : (size_t)0);
     p->slab_bytes = slab_band * (size_t)p->ws_bands;
     p->ws_bytes = (size_t)S * n3 * elem * p->ws_bands + p->slab_bytes + (size_t)N * sizeof(double) * (1 + p->ngroups);
     if ((e = dmalloc((void**)&p->d_cyl, (size_t)S * n3 * elem * p->ws_bands))) { free_plan(p); return cuda_fail(e, "cudaMalloc(cylinder)"); }
@@ -896,6 +903,19 @@ int vloc_plan_create(vloc_plan* out, int n1, int n2, int n3, const int32_t* g, i
     if ((e = cudaStreamSynchronize(st))) { free_plan(p); return cuda_fail(e, "plan create sync"); }
     *out = p;
     return VLOC_OK;
+}
+
+extern "C" {
+
+int vloc_plan_create(vloc_plan* out, int n1, int n2, int n3, const int32_t* g, int64_t npw, int flags,
+                     int64_t max_bands_per_chunk, void* stream) {
+    if (!out) return VLOC_ERR_ARG;
+    *out = nullptr;
+    bool grew = false;
+    const int rc = create_plan(out, n1, n2, n3, g, npw, flags, max_bands_per_chunk, stream, true, &grew);
+    // a chunk that fits with the slab but not with the dense rows: the five launches
+    if (rc != VLOC_ERR_ALLOC || !grew) return rc;
+    return create_plan(out, n1, n2, n3, g, npw, flags, max_bands_per_chunk, stream, false, &grew);
 }
 
 int vloc_plan_set_schedule(vloc_plan p, int axis, int nst, const int32_t* radix) {

@@ -10,19 +10,22 @@
 
 #define MAXF 4096
 #define MAXL 65536
+#define MAXM 4096
 
 static int g_dev = 0;
 static size_t g_free = (size_t)270 << 30, g_alloc = 0;
 static uintptr_t g_next = (uintptr_t)1 << 40, g_handle = 4096;
 static struct { const void* f; int dev; int bytes; } g_lim[MAXF];
 static int g_nlim = 0;
+static struct { uintptr_t at; size_t bytes; } g_mem[MAXM];
+static int g_nmem = 0;
 static uintptr_t g_launch[MAXL];   /* stream of each launch */
 static int g_nlaunch = 0;
 static cudaError_t g_last = cudaSuccess;
 
 /* ---- controls of the test */
 void fake_set_device(int d) { g_dev = d; }
-void fake_set_free(size_t b) { g_free = b; }
+void fake_set_free(size_t b) { g_free = g_alloc + b; }
 size_t fake_allocated(void) { return g_alloc; }
 int fake_limits(void) { return g_nlim; }   /* cudaFuncSetAttribute calls that raised a limit */
 int fake_launches(void) { return g_nlaunch; }
@@ -58,13 +61,19 @@ cudaError_t __cudaLaunchKernel(const void* k, struct dim3 g, struct dim3 b, void
     return launched(k, smem, st);
 }
 cudaError_t cudaMalloc(void** p, size_t n) {
+    if (n > g_free - g_alloc || g_nmem == MAXM) return g_last = cudaErrorMemoryAllocation;
     *p = (void*)g_next;
+    g_mem[g_nmem].at = g_next; g_mem[g_nmem++].bytes = n;
     g_next += (n + 511) / 256 * 256;
     g_alloc += n;
     return cudaSuccess;
 }
-cudaError_t cudaFree(void* p) { (void)p; return cudaSuccess; }
-cudaError_t cudaMemGetInfo(size_t* f, size_t* t) { *f = g_free; *t = g_free; return cudaSuccess; }
+cudaError_t cudaFree(void* p) {
+    for (int i = 0; p && i < g_nmem; ++i)
+        if (g_mem[i].at == (uintptr_t)p) { g_alloc -= g_mem[i].bytes; g_mem[i] = g_mem[--g_nmem]; return cudaSuccess; }
+    return p ? (g_last = cudaErrorInvalidValue) : cudaSuccess;
+}
+cudaError_t cudaMemGetInfo(size_t* f, size_t* t) { *f = g_free - g_alloc; *t = g_free; return cudaSuccess; }
 cudaError_t cudaMemcpy(void* d, const void* s, size_t n, enum cudaMemcpyKind k) { (void)d; (void)s; (void)n; (void)k; return cudaSuccess; }
 cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, enum cudaMemcpyKind k, cudaStream_t st) {
     (void)d; (void)s; (void)n; (void)k; (void)st;

@@ -87,3 +87,57 @@ done(res)
     assert [r[0] for r in out] == [[0] * 4] * 3
     assert out[0][1] == out[1][1]      # the second device as the first
     assert out[2][1] == 0 and [r[2] for r in out] == [0] * 3
+
+
+@pytest.mark.parametrize("flags", ["VLOC_F32", "VLOC_F64", "VLOC_F32 | vloc.VLOC_GAMMA"])
+@pytest.mark.parametrize("n,r", [((144, 144, 144), 3), ((144, 144, 144), 9), ((96, 96, 96), 5), ((128, 100, 96), 6.5),
+                                 ((96, 96, 96), 24), ((144, 144, 144), 36), ((54, 54, 54), 13), ((48, 48, 48), 2)])
+def test_automatic_chunk_keeps_the_documented_workspace(run, n, r, flags):
+    """max_bands_per_chunk <= 0: the per-band workspace of a chunk (cylinder,
+    and slab or dense rows) stays within 6 GiB and a sixteenth of the free
+    memory, whatever the sphere; the V / density accumulators and the Gamma
+    buffers are apart."""
+    out = run(f"""
+res = []
+for free in (270 << 30, 24 << 30):
+    rt.fake_set_free(free)
+    h = plan({n!r}, {r}, vloc.{flags})
+    i = info(h)
+    res.append([free, i.chunk_bands, i.workspace_bytes, i.npw])
+done(res)
+""")
+    N = n[0] * n[1] * n[2]
+    elem = 16 if "F64" in flags else 8
+    for free, chunk, ws, npw in out:
+        groups = (max(1, max(chunk, 2) // 2) + 15) // 16
+        ws -= N * 8 * (1 + groups)
+        if "GAMMA" in flags:
+            ws -= 2 * chunk * (2 * npw - 1) * elem    # G = 0 is its own mirror
+        assert 1 <= chunk <= 2048
+        assert ws <= min(6 << 30, free // 16)
+        assert ws * (chunk + 1) > min(6 << 30, free // 16) * chunk or chunk == 2048    # and uses it
+
+
+def test_given_chunk_that_does_not_fit_with_the_dense_rows(run):
+    """A small sphere on a large grid with a chunk sized by the caller: where
+    the dense rows of the three-launch form do not fit, the plan is made for
+    five launches; where not even the slab does, the call fails."""
+    out = run("""
+def create(free):
+    rt.fake_set_free(free)
+    g = np.ascontiguousarray(synth.sphere_glist(96, 96, 96, 4), dtype=np.int32)
+    h = ctypes.c_void_p()
+    rc = lib.vloc_plan_create(ctypes.byref(h), 96, 96, 96, g.ctypes.data_as(ctypes.POINTER(ctypes.c_int32)), len(g),
+                              vloc.VLOC_F32, 1024, None)
+    if rc:
+        return [rc, None, None]
+    n0 = rt.fake_launches()
+    rcs = [lib.vloc_apply(h, addr(0), addr(1), 64, addr(2), None), lib.vloc_density(h, addr(0), None, 64, addr(3), None)]
+    ws = info(h).workspace_bytes
+    return [rc, rcs, ws, lib.vloc_plan_destroy(h)]
+done([create(8 << 30), create(2 << 30), create(256 << 20), [rt.cudaGetLastError(), rt.fake_allocated()]])
+""")
+    assert out[0][:2] == [0, [0, 0]] and out[1][:2] == [0, [0, 0]]
+    assert out[1][2] <= 2 << 30 and out[1][2] <= out[0][2]
+    assert out[2][0] == -4    # VLOC_ERR_ALLOC
+    assert out[3] == [0, 0]    # nothing leaks, and the failures leave no error behind
