@@ -1478,17 +1478,19 @@ int vloc_density(vloc_plan p, const void* c, const void* occ, int64_t nb, void* 
     return launch(p, KK_AUX, st, [&] { return launch_finish_grad_v(dbl, p->d_acc, rho, p->N, st); });
 }
 
-// Whether an instance of a batch should not share the GPU with another length's
-// y/x pass.  Two such kernels on an SM evict each other's code from its
+// Whether an instance of a batch runs the y/x pass and should not share the GPU
+// with another length's.  Two such kernels on an SM evict each other's code from its
 // instruction cache: eight cubes 48^3..144^3 with 64..512 bands took 18.2 ms on
 // parallel branches and 16.7 one after another, with 4..32 bands 1.21 and 1.14;
 // 96^3 + 100^3 x 128 1.116 / 1.055; 90^3, 96^3, 108^3 x 100 1.32 / 1.22.  It is
 // the other way round where the kernels are the same (4 x 64 bands at 144^3 3.84
 // / 3.96) or short (60^3, 64^3, 72^3 x 256 0.827 / 0.857), and where the
 // instances do not fill the GPU (eight of 96^3 x 8 0.178 / 0.236; the count is
-// bands x z rows x y columns, the eight cubes with 4..32 bands lose from 800 k on).
+// complex bands x z rows x y columns, the eight cubes with 4..32 bands lose from
+// 800 k on).
 static bool batch_apart(vloc_plan p, int64_t nb) {
-    return p->line_on && nb * p->n3 * p->n2 >= 400000 && p->n1 + p->n2 >= 180;
+    const int64_t m = p->gamma ? (nb + 1) / 2 : nb;  // the bands of the y/x pass
+    return line_chunk(p, std::min<int64_t>(p->chunk, m)) && m * p->n3 * p->n2 >= 400000 && p->n1 + p->n2 >= 180;
 }
 
 int vloc_apply_batched(int ninst, const vloc_plan* plans, const void* const* c, const void* const* V,

@@ -141,3 +141,22 @@ done([create(8 << 30), create(2 << 30), create(256 << 20), [rt.cudaGetLastError(
     assert out[1][2] <= 2 << 30 and out[1][2] <= out[0][2]
     assert out[2][0] == -4    # VLOC_ERR_ALLOC
     assert out[3] == [0, 0]    # nothing leaks, and the failures leave no error behind
+
+
+# Two large instances of different lengths: in turn on one branch if both run
+# the fused y/x pass on enough complex bands, else on two branches.
+@pytest.mark.parametrize("bands,flags,chunk,branches", [
+    (60, "VLOC_F32", 0, 1), (30, "VLOC_F32", 0, 2), (200, "VLOC_F32", 2, 2),    # chunk 2: five launches
+    (60, "VLOC_F32 | vloc.VLOC_GAMMA", 0, 2), (120, "VLOC_F32 | vloc.VLOC_GAMMA", 0, 1),    # 30 and 60 pairs
+    (60, "VLOC_F64", 0, 2)])
+def test_batch_instances_in_turn_or_on_branches(run, bands, flags, chunk, branches):
+    out = run(f"""
+hs = [plan((n,) * 3, n / 4, vloc.{flags} | vloc.VLOC_GRAPH, {chunk}) for n in (96, 100)]
+n0 = rt.fake_launches()
+vp = ctypes.c_void_p * 2
+rc = lib.vloc_apply_batched(2, vp(*hs), vp(addr(0), addr(1)), vp(addr(2), addr(3)), (ctypes.c_int64 * 2)({bands}, {bands}),
+                            vp(addr(4), addr(5)), None)
+done([rc, [rt.fake_launch_stream(i) for i in range(n0, rt.fake_launches())]])
+""")
+    assert out[0] == 0
+    assert len(set(out[1])) == branches and 0 not in out[1]
