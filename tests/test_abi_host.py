@@ -277,3 +277,17 @@ def test_gamma_partition_deals_mirror_pairs(lib, n, R):
     for r, i in enumerate(pairs):
         want[i] = want[mirror[i]] = r % P2
     assert np.array_equal(part, want)
+
+
+def test_current_stream_without_the_private_accessor(monkeypatch):
+    """The binding takes the current stream's handle from a name inside
+    torch._C; a torch without it gives the same through the public call."""
+    torch = pytest.importorskip("torch")
+    import types
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 3)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda *a: types.SimpleNamespace(cuda_stream=77))
+    monkeypatch.setattr(torch._C, "_cuda_getCurrentRawStream", lambda d: 70 + d, raising=False)
+    assert vloc._stream_ptr() == 73
+    assert vloc._stream_ptr(types.SimpleNamespace(cuda_stream=5)) == 5
+    monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream")
+    assert vloc._stream_ptr() == 77
