@@ -16,6 +16,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <numeric>
@@ -34,6 +35,14 @@ thread_local char g_last_cuda[256] = "";
 int cuda_fail(cudaError_t e, const char* what) {
     snprintf(g_last_cuda, sizeof(g_last_cuda), "%s: %s", what, cudaGetErrorString(e));
     return e == cudaErrorMemoryAllocation ? VLOC_ERR_ALLOC : VLOC_ERR_CUDA;
+}
+// f() for a C entry point: host memory that runs out is an error code there.
+template <class F> int guarded(F&& f) {
+    try {
+        return f();
+    } catch (const std::bad_alloc&) {
+        return VLOC_ERR_ALLOC;
+    }
 }
 #define CK(call)                                              \
     do {                                                      \
@@ -439,7 +448,9 @@ static int create_plan(vloc_plan* out, int n1, int n2, int n3, const int32_t* g,
 
     const FaultSpec fault = fault_spec();
     int alloc_no = 0;  // allocations so far (fault injection counts them)
-    vloc_plan p = fault.alloc_at == alloc_no++ ? nullptr : new (std::nothrow) vloc_plan_s();
+    std::unique_ptr<vloc_plan_s, void (*)(vloc_plan)> own(
+        fault.alloc_at == alloc_no++ ? nullptr : new (std::nothrow) vloc_plan_s(), free_plan);
+    const vloc_plan p = own.get();
     if (!p) return VLOC_ERR_ALLOC;
     auto dmalloc = [&](void** ptr, size_t bytes) -> cudaError_t {
         if (fault.alloc_at == alloc_no++) return cudaErrorMemoryAllocation;
@@ -456,7 +467,7 @@ static int create_plan(vloc_plan* out, int n1, int n2, int n3, const int32_t* g,
     p->df = (flags & VLOC_DOUBLE_FLOAT) && !(flags & VLOC_GENERIC_KERNELS) && has_df(n1) && has_df(n2) && has_df(n3);
     for (int a = 0; a < 3; ++a) {
         p->ax.n[a] = ns[a];
-        if (!plan_radices(ns[a], &p->ax.nst[a], p->ax.radix[a])) { free_plan(p); return VLOC_ERR_SIZE; }
+        if (!plan_radices(ns[a], &p->ax.nst[a], p->ax.radix[a])) return VLOC_ERR_SIZE;
     }
 
     // ---- index map and validation (Eqs. 2-3)
@@ -465,9 +476,9 @@ static int create_plan(vloc_plan* out, int n1, int n2, int n3, const int32_t* g,
         std::vector<unsigned char> seen((size_t)N, 0);
         for (int64_t q = 0; q < npw; ++q) {
             const int h = g[3 * q], k = g[3 * q + 1], l = g[3 * q + 2];
-            if (!valid_miller(h, n1) || !valid_miller(k, n2) || !valid_miller(l, n3)) { free_plan(p); return VLOC_ERR_GLIST; }
+            if (!valid_miller(h, n1) || !valid_miller(k, n2) || !valid_miller(l, n3)) return VLOC_ERR_GLIST;
             const long long j = ((long long)pmod(h, n1) * n2 + pmod(k, n2)) * n3 + pmod(l, n3);
-            if (seen[(size_t)j]) { free_plan(p); return VLOC_ERR_GLIST; }
+            if (seen[(size_t)j]) return VLOC_ERR_GLIST;
             seen[(size_t)j] = 1;
             p->grid_index[q] = j;
         }
@@ -768,7 +779,7 @@ static int create_plan(vloc_plan* out, int n1, int n2, int n3, const int32_t* g,
 
     if (host_only) {
         p->chunk = 0;
-        *out = p;
+        *out = own.release();
         return VLOC_OK;
     }
     // ---- tables of the line path (not among the host tables: the
@@ -780,27 +791,27 @@ static int create_plan(vloc_plan* out, int n1, int n2, int n3, const int32_t* g,
     // shared-memory budget of the largest kernel tile
     int dev = 0;
     cudaError_t e;
-    if ((e = cudaGetDevice(&dev))) { free_plan(p); return cuda_fail(e, "cudaGetDevice"); }
+    if ((e = cudaGetDevice(&dev))) return cuda_fail(e, "cudaGetDevice");
     p->device = dev;
     int maxopt = 0;
     if ((e = cudaDeviceGetAttribute(&maxopt, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev))) {
-        free_plan(p); return cuda_fail(e, "cudaDeviceGetAttribute");
+        return cuda_fail(e, "cudaDeviceGetAttribute");
     }
-    if (smem_bytes_for(dbl, nmax) > (size_t)maxopt) { free_plan(p); return VLOC_ERR_SIZE; }
+    if (smem_bytes_for(dbl, nmax) > (size_t)maxopt) return VLOC_ERR_SIZE;
     p->smem_optin = maxopt;
 
     // ---- device tables (one allocation)
     cudaStream_t st = (cudaStream_t)stream;
     const std::vector<int>& blob = p->host_tables;
-    if ((e = dmalloc((void**)&p->d_tables, blob.size() * sizeof(int)))) { free_plan(p); return cuda_fail(e, "cudaMalloc(tables)"); }
+    if ((e = dmalloc((void**)&p->d_tables, blob.size() * sizeof(int)))) return cuda_fail(e, "cudaMalloc(tables)");
     if ((e = cudaMemcpyAsync(p->d_tables, blob.data(), blob.size() * sizeof(int), cudaMemcpyHostToDevice, st))) {
-        free_plan(p); return cuda_fail(e, "upload tables");
+        return cuda_fail(e, "upload tables");
     }
     p->dt = device_tables(p->d_tables, p->lay, n1, n2, n3, npw);
     if (lh.cls >= 0) {
-        if ((e = dmalloc(&p->d_line, lh.blob.size() * sizeof(int)))) { free_plan(p); return cuda_fail(e, "cudaMalloc(line tables)"); }
+        if ((e = dmalloc(&p->d_line, lh.blob.size() * sizeof(int)))) return cuda_fail(e, "cudaMalloc(line tables)");
         if ((e = cudaMemcpyAsync(p->d_line, lh.blob.data(), lh.blob.size() * sizeof(int), cudaMemcpyHostToDevice, st))) {
-            free_plan(p); return cuda_fail(e, "upload line tables");
+            return cuda_fail(e, "upload line tables");
         }
         const int* base = (const int*)p->d_line;
         line::Tables& t = p->lt;
@@ -818,20 +829,20 @@ static int create_plan(vloc_plan* out, int n1, int n2, int n3, const int32_t* g,
 
     // ---- twiddles exp(+2 pi i j / n), FP64-made
     for (int a = 0; a < 3; ++a) {
-        if ((e = dmalloc((void**)&p->d_tw[a], (size_t)ns[a] * elem))) { free_plan(p); return cuda_fail(e, "cudaMalloc(twiddles)"); }
-        if (launch_twiddles(dbl, p->d_tw[a], ns[a], st)) { free_plan(p); return cuda_fail(cudaGetLastError(), "twiddles"); }
+        if ((e = dmalloc((void**)&p->d_tw[a], (size_t)ns[a] * elem))) return cuda_fail(e, "cudaMalloc(twiddles)");
+        if (launch_twiddles(dbl, p->d_tw[a], ns[a], st)) return cuda_fail(cudaGetLastError(), "twiddles");
     }
-    if ((e = (cudaError_t)set_smem_limits(dbl, nmax, maxopt))) { free_plan(p); return cuda_fail(e, "cudaFuncSetAttribute"); }
-    if ((e = dmalloc((void**)&p->d_err, sizeof(int)))) { free_plan(p); return cuda_fail(e, "cudaMalloc(error flag)"); }
+    if ((e = (cudaError_t)set_smem_limits(dbl, nmax, maxopt))) return cuda_fail(e, "cudaFuncSetAttribute");
+    if ((e = dmalloc((void**)&p->d_err, sizeof(int)))) return cuda_fail(e, "cudaMalloc(error flag)");
 
-    if ((e = cudaMemsetAsync(p->d_err, 0, sizeof(int), st))) { free_plan(p); return cuda_fail(e, "clear error flag"); }
+    if ((e = cudaMemsetAsync(p->d_err, 0, sizeof(int), st))) return cuda_fail(e, "clear error flag");
     p->dt.err = p->d_err;
     if (p->df) {
         for (int a = 0; a < 3; ++a) {
-            if ((e = dmalloc((void**)&p->d_twdf[a], (size_t)ns[a] * 32))) { free_plan(p); return cuda_fail(e, "cudaMalloc(df twiddles)"); }
-            if (launch_twiddles_df(p->d_tw[a], p->d_twdf[a], ns[a], st)) { free_plan(p); return cuda_fail(cudaGetLastError(), "df twiddles"); }
+            if ((e = dmalloc((void**)&p->d_twdf[a], (size_t)ns[a] * 32))) return cuda_fail(e, "cudaMalloc(df twiddles)");
+            if (launch_twiddles_df(p->d_tw[a], p->d_twdf[a], ns[a], st)) return cuda_fail(cudaGetLastError(), "df twiddles");
         }
-        if ((e = dmalloc((void**)&p->d_vdf, (size_t)N * 8))) { free_plan(p); return cuda_fail(e, "cudaMalloc(df V)"); }
+        if ((e = dmalloc((void**)&p->d_vdf, (size_t)N * 8))) return cuda_fail(e, "cudaMalloc(df V)");
     }
 
     // ---- workspace: cylinder [chunk][S][n3] + slab [chunk][NP][n2][n3], whose
@@ -859,14 +870,14 @@ static int create_plan(vloc_plan* out, int n1, int n2, int n3, const int32_t* g,
     p->ngroups = (int)((std::max<long long>(1, p->ws_bands / 2) + kGradBandsPerGroup - 1) / kGradBandsPerGroup);
     p->slab_bytes = slab_band * (size_t)p->ws_bands;
     p->ws_bytes = (size_t)S * n3 * elem * p->ws_bands + p->slab_bytes + (size_t)N * sizeof(double) * (1 + p->ngroups);
-    if ((e = dmalloc((void**)&p->d_cyl, (size_t)S * n3 * elem * p->ws_bands))) { free_plan(p); return cuda_fail(e, "cudaMalloc(cylinder)"); }
-    if ((e = dmalloc((void**)&p->d_slab, p->slab_bytes))) { free_plan(p); return cuda_fail(e, "cudaMalloc(slab)"); }
+    if ((e = dmalloc((void**)&p->d_cyl, (size_t)S * n3 * elem * p->ws_bands))) return cuda_fail(e, "cudaMalloc(cylinder)");
+    if ((e = dmalloc((void**)&p->d_slab, p->slab_bytes))) return cuda_fail(e, "cudaMalloc(slab)");
     if (p->gamma) {
-        if ((e = dmalloc((void**)&p->d_gamma_neg, sizeof(int) * (size_t)npw_user))) { free_plan(p); return cuda_fail(e, "cudaMalloc(gamma map)"); }
+        if ((e = dmalloc((void**)&p->d_gamma_neg, sizeof(int) * (size_t)npw_user))) return cuda_fail(e, "cudaMalloc(gamma map)");
         if ((e = cudaMemcpyAsync(p->d_gamma_neg, gamma_neg.data(), sizeof(int) * (size_t)npw_user, cudaMemcpyHostToDevice, st))) {
-            free_plan(p); return cuda_fail(e, "upload gamma map");
+            return cuda_fail(e, "upload gamma map");
         }
-        if ((e = dmalloc((void**)&p->d_gamma_buf, 2 * (size_t)p->chunk * npw * elem))) { free_plan(p); return cuda_fail(e, "cudaMalloc(gamma buffers)"); }
+        if ((e = dmalloc((void**)&p->d_gamma_buf, 2 * (size_t)p->chunk * npw * elem))) return cuda_fail(e, "cudaMalloc(gamma buffers)");
         p->ws_bytes += 2 * (size_t)p->chunk * npw * elem;
     }
     // tensor map over the slab workspace for the persistent TMA x-pass (FP32,
@@ -899,9 +910,9 @@ static int create_plan(vloc_plan* out, int n1, int n2, int n3, const int32_t* g,
 
     // dL/dV accumulator [N] followed by the band groups' partial sums [ngroups][N]
     // (the line path's transposed V, N floats, shares it)
-    if ((e = dmalloc((void**)&p->d_acc, (size_t)N * sizeof(double) * (1 + p->ngroups)))) { free_plan(p); return cuda_fail(e, "cudaMalloc(acc)"); }
-    if ((e = cudaStreamSynchronize(st))) { free_plan(p); return cuda_fail(e, "plan create sync"); }
-    *out = p;
+    if ((e = dmalloc((void**)&p->d_acc, (size_t)N * sizeof(double) * (1 + p->ngroups)))) return cuda_fail(e, "cudaMalloc(acc)");
+    if ((e = cudaStreamSynchronize(st))) return cuda_fail(e, "plan create sync");
+    *out = own.release();
     return VLOC_OK;
 }
 
@@ -912,10 +923,14 @@ int vloc_plan_create(vloc_plan* out, int n1, int n2, int n3, const int32_t* g, i
     if (!out) return VLOC_ERR_ARG;
     *out = nullptr;
     bool grew = false;
-    const int rc = create_plan(out, n1, n2, n3, g, npw, flags, max_bands_per_chunk, stream, true, &grew);
+    auto create = [&](bool line_path) {
+        return guarded([&] {
+            return create_plan(out, n1, n2, n3, g, npw, flags, max_bands_per_chunk, stream, line_path, &grew);
+        });
+    };
+    const int rc = create(true);
     // a chunk that fits with the slab but not with the dense rows: the five launches
-    if (rc != VLOC_ERR_ALLOC || !grew) return rc;
-    return create_plan(out, n1, n2, n3, g, npw, flags, max_bands_per_chunk, stream, false, &grew);
+    return rc == VLOC_ERR_ALLOC && grew ? create(false) : rc;
 }
 
 int vloc_plan_set_schedule(vloc_plan p, int axis, int nst, const int32_t* radix) {
@@ -1182,6 +1197,12 @@ static int graph_run(vloc_plan owner, const std::vector<vloc_plan>& plans, std::
         return cuda_fail(e, "capture stream");
     std::vector<long long> l0;
     std::vector<bool> prof;
+    vloc_plan_s::GraphEntry ent;
+    // what grows after the profiling flags are off and the capture is open must not throw
+    l0.reserve(plans.size());
+    prof.reserve(plans.size());
+    ent.kernels.reserve(plans.size());
+    owner->graphs.reserve(8);
     for (vloc_plan q : plans) {
         l0.push_back(q->launches);
         prof.push_back(q->prof_on);
@@ -1194,11 +1215,10 @@ static int graph_run(vloc_plan owner, const std::vector<vloc_plan>& plans, std::
         restore();
         return cuda_fail(e, "cudaStreamBeginCapture");
     }
-    const int rc = enqueue(owner->cap_stream);
+    const int rc = guarded([&] { return enqueue(owner->cap_stream); });
     cudaGraph_t graph = nullptr;
     e = cudaStreamEndCapture(owner->cap_stream, &graph);
     restore();
-    vloc_plan_s::GraphEntry ent;
     for (size_t i = 0; i < plans.size(); ++i) {
         ent.kernels.push_back({plans[i], plans[i]->launches - l0[i]});
         plans[i]->launches = l0[i];
@@ -1231,8 +1251,10 @@ int vloc_apply(vloc_plan p, const void* c, const void* V, int64_t nb, void* out,
     int rc = check_io(p, c, V, nb, out);
     if (rc || nb == 0) return rc;
     if (p->flags & VLOC_GRAPH)
-        return graph_run(p, {p}, {(uintptr_t)c, (uintptr_t)V, (uintptr_t)nb, (uintptr_t)out}, (cudaStream_t)stream,
-                         [&](cudaStream_t cs) { return apply_any(p, c, V, nb, out, cs); });
+        return guarded([&] {
+            return graph_run(p, {p}, {(uintptr_t)c, (uintptr_t)V, (uintptr_t)nb, (uintptr_t)out}, (cudaStream_t)stream,
+                             [&](cudaStream_t cs) { return apply_any(p, c, V, nb, out, cs); });
+        });
     return apply_any(p, c, V, nb, out, (cudaStream_t)stream);
 }
 
@@ -1244,8 +1266,11 @@ int vloc_apply_h(vloc_plan p, const void* c, const void* V, const void* diag, in
     if (!aligned(diag, re)) return VLOC_ERR_ARG;
     if (overlap(diag, (size_t)p->npw_user * re, out, (size_t)nb * p->npw_user * p->elem)) return VLOC_ERR_ARG;
     if (p->flags & VLOC_GRAPH)
-        return graph_run(p, {p}, {(uintptr_t)c, (uintptr_t)V, (uintptr_t)nb, (uintptr_t)out, (uintptr_t)diag},
-                         (cudaStream_t)stream, [&](cudaStream_t cs) { return apply_any(p, c, V, nb, out, cs, diag); });
+        return guarded([&] {
+            return graph_run(p, {p}, {(uintptr_t)c, (uintptr_t)V, (uintptr_t)nb, (uintptr_t)out, (uintptr_t)diag},
+                             (cudaStream_t)stream,
+                             [&](cudaStream_t cs) { return apply_any(p, c, V, nb, out, cs, diag); });
+        });
     return apply_any(p, c, V, nb, out, (cudaStream_t)stream, diag);
 }
 
@@ -1493,8 +1518,8 @@ static bool batch_apart(vloc_plan p, int64_t nb) {
     return line_chunk(p, std::min<int64_t>(p->chunk, m)) && m * p->n3 * p->n2 >= 400000 && p->n1 + p->n2 >= 180;
 }
 
-int vloc_apply_batched(int ninst, const vloc_plan* plans, const void* const* c, const void* const* V,
-                       const int64_t* nb, void* const* out, void* stream) {
+static int apply_batched(int ninst, const vloc_plan* plans, const void* const* c, const void* const* V,
+                         const int64_t* nb, void* const* out, void* stream) {
     if (ninst < 0 || (ninst > 0 && (!plans || !c || !V || !nb || !out))) return VLOC_ERR_ARG;
     for (int i = 0; i < ninst; ++i) {
         if (!plans[i] || plans[i]->dbl != plans[0]->dbl) return VLOC_ERR_ARG;
@@ -1520,6 +1545,8 @@ int vloc_apply_batched(int ninst, const vloc_plan* plans, const void* const* c, 
     vloc_plan owner = plans[0];
     const int K = std::min(ninst, (int)kBatchBranches);
     cudaError_t e;
+    owner->branch_streams.reserve(kBatchBranches);
+    owner->branch_events.reserve(kBatchBranches);
     while ((int)owner->branch_streams.size() < K) {
         cudaStream_t s;
         if ((e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking))) return cuda_fail(e, "branch stream");
@@ -1589,6 +1616,10 @@ int vloc_apply_batched(int ninst, const vloc_plan* plans, const void* const* c, 
         if (std::find(ps.begin(), ps.end(), plans[i]) == ps.end()) ps.push_back(plans[i]);
     }
     return graph_run(plans[0], ps, std::move(key), (cudaStream_t)stream, branched);
+}
+int vloc_apply_batched(int ninst, const vloc_plan* plans, const void* const* c, const void* const* V,
+                       const int64_t* nb, void* const* out, void* stream) {
+    return guarded([&] { return apply_batched(ninst, plans, c, V, nb, out, stream); });
 }
 
 // Host-buffer apply; `blocking`: synchronise before return, otherwise leave

@@ -20,7 +20,7 @@ static int g_nlim = 0;
 static struct { uintptr_t at; size_t bytes; } g_mem[MAXM];
 static int g_nmem = 0;
 static uintptr_t g_launch[MAXL];   /* stream of each launch */
-static int g_nlaunch = 0;
+static int g_nlaunch = 0, g_cap = 0;
 static cudaError_t g_last = cudaSuccess;
 
 /* ---- controls of the test */
@@ -28,6 +28,7 @@ void fake_set_device(int d) { g_dev = d; }
 void fake_set_free(size_t b) { g_free = g_alloc + b; }
 size_t fake_allocated(void) { return g_alloc; }
 int fake_limits(void) { return g_nlim; }   /* cudaFuncSetAttribute calls that raised a limit */
+int fake_captures(void) { return g_cap; }   /* begun and not ended */
 int fake_launches(void) { return g_nlaunch; }
 uintptr_t fake_launch_stream(int i) { return g_launch[i]; }
 
@@ -106,8 +107,8 @@ cudaError_t cudaEventDestroy(cudaEvent_t e) { (void)e; return cudaSuccess; }
 cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t s) { (void)e; (void)s; return cudaSuccess; }
 cudaError_t cudaEventSynchronize(cudaEvent_t e) { (void)e; return cudaSuccess; }
 cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t a, cudaEvent_t b) { (void)a; (void)b; *ms = 0.f; return cudaSuccess; }
-cudaError_t cudaStreamBeginCapture(cudaStream_t s, enum cudaStreamCaptureMode m) { (void)s; (void)m; return cudaSuccess; }
-cudaError_t cudaStreamEndCapture(cudaStream_t s, cudaGraph_t* g) { (void)s; *g = (cudaGraph_t)(g_handle += 16); return cudaSuccess; }
+cudaError_t cudaStreamBeginCapture(cudaStream_t s, enum cudaStreamCaptureMode m) { (void)s; (void)m; ++g_cap; return cudaSuccess; }
+cudaError_t cudaStreamEndCapture(cudaStream_t s, cudaGraph_t* g) { (void)s; --g_cap; *g = (cudaGraph_t)(g_handle += 16); return cudaSuccess; }
 cudaError_t cudaGraphInstantiate(cudaGraphExec_t* x, cudaGraph_t g, unsigned long long fl) {
     (void)g; (void)fl;
     *x = (cudaGraphExec_t)(g_handle += 16);

@@ -42,6 +42,23 @@ def done(x):
     print("RESULT " + json.dumps(x))
 """ % ROOT
 
+# operator new of the child: allocation number fake_new_at (counted from the
+# call of that function) throws, with no memory to spare.
+NEW = """
+#include <cstdlib>
+#include <new>
+static long g_left = -1;
+extern "C" void fake_new_at(long k) { g_left = k; }
+void* operator new(std::size_t n) {
+    if (g_left == 0) throw std::bad_alloc();
+    if (g_left > 0) --g_left;
+    if (void* p = std::malloc(n ? n : 1)) return p;
+    throw std::bad_alloc();
+}
+void operator delete(void* p) noexcept { std::free(p); }
+void operator delete(void* p, std::size_t) noexcept { std::free(p); }
+"""
+
 
 @pytest.fixture(scope="module")
 def run(tmp_path_factory):
@@ -49,12 +66,15 @@ def run(tmp_path_factory):
     if not sys.platform.startswith("linux") or shutil.which("gcc") is None:
         pytest.skip("needs gcc and LD_PRELOAD")
     build.build()
-    so = str(tmp_path_factory.mktemp("fake") / "libfake_cudart.so")
+    tmp = tmp_path_factory.mktemp("fake")
+    so, new = str(tmp / "libfake_cudart.so"), str(tmp / "libfake_new.so")
     subprocess.check_call(["gcc", "-shared", "-fPIC", "-O1", "-Wno-builtin-declaration-mismatch",
                            "-I" + os.path.join(build._cuda_home(), "include"), "-o", so, os.path.join(HERE, "fake_cudart.c")])
+    (tmp / "new.cpp").write_text(NEW)
+    subprocess.check_call(["g++", "-shared", "-fPIC", "-O1", "-o", new, str(tmp / "new.cpp")])
 
     def child(code):
-        env = dict(os.environ, LD_PRELOAD=so)
+        env = dict(os.environ, LD_PRELOAD=so + ":" + new)
         p = subprocess.run([sys.executable, "-c", CHILD + code], env=env, capture_output=True, text=True, timeout=300)
         assert p.returncode == 0, p.stdout + p.stderr
         return json.loads([ln for ln in p.stdout.splitlines() if ln.startswith("RESULT ")][-1][7:])
@@ -160,3 +180,48 @@ done([rc, [rt.fake_launch_stream(i) for i in range(n0, rt.fake_launches())]])
 """)
     assert out[0] == 0
     assert len(set(out[1])) == branches and 0 not in out[1]
+
+
+@pytest.mark.parametrize("flags", ["VLOC_F32", "VLOC_F32 | vloc.VLOC_GAMMA", "VLOC_F64", "VLOC_F32 | vloc.VLOC_HOST_ONLY"])
+def test_host_memory_that_runs_out_in_plan_creation_is_an_error_code(run, flags):
+    """Every host allocation of vloc_plan_create fails in turn (from that one
+    on): the call returns VLOC_ERR_ALLOC, frees what it had, and no exception
+    reaches the caller."""
+    out = run(f"""
+n, flags = (24, 24, 24), vloc.{flags}
+g = synth.sphere_glist(*n, 6)
+g = np.ascontiguousarray(synth.half_sphere(g) if flags & vloc.VLOC_GAMMA else g, dtype=np.int32)
+gp = g.ctypes.data_as(ctypes.POINTER(ctypes.c_int32))
+codes, k = [], 0
+while True:
+    h = ctypes.c_void_p()
+    rt.fake_new_at(k)
+    rc = lib.vloc_plan_create(ctypes.byref(h), *n, gp, len(g), flags, 0, None)
+    rt.fake_new_at(-1)
+    codes.append(rc)
+    if rc == 0:
+        break
+    assert not h.value and rt.fake_allocated() == 0
+    k = k + 1 if k < 60 else k + 1 + k // 8
+done([codes[:-1], lib.vloc_plan_destroy(h), rt.fake_allocated()])
+""")
+    assert len(out[0]) > 20 and set(out[0]) == {-4}
+    assert out[1:] == [0, 0]
+
+
+def test_host_memory_that_runs_out_in_a_captured_batch_is_an_error_code(run):
+    out = run("""
+hs = [plan((n,) * 3, n / 4, vloc.VLOC_F32 | vloc.VLOC_GRAPH) for n in (48, 60, 48)]
+vp = ctypes.c_void_p * 3
+args = (3, vp(*hs), vp(addr(0), addr(1), addr(2)), vp(addr(3), addr(4), addr(5)), (ctypes.c_int64 * 3)(20, 20, 20),
+        vp(addr(6), addr(7), addr(8)), None)
+codes, k = [], 0
+while not codes or codes[-1]:
+    rt.fake_new_at(k)
+    codes.append(lib.vloc_apply_batched(*args))
+    rt.fake_new_at(-1)
+    k += 1
+done([codes, rt.fake_captures()])
+""")
+    assert len(out[0]) > 5 and set(out[0][:-1]) == {-4} and out[0][-1] == 0
+    assert out[1] == 0    # every capture that was begun was ended
