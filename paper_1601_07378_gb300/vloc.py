@@ -157,8 +157,10 @@ def _stream_ptr(stream=None) -> int:
     if stream is not None:
         return stream.cuda_stream
     import torch
-    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)  # not a public name
-    return raw(torch.cuda.current_device()) if raw else torch.cuda.current_stream().cuda_stream
+    try:
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    except AttributeError:  # not a public name
+        return torch.cuda.current_stream().cuda_stream
 
 
 def _ptr(t) -> int:
