@@ -121,7 +121,7 @@ int launch_twiddles_df(const void* tw64, void* twdf, int n, cudaStream_t st) {
     k_twiddles_df<<<(n + 127) / 128, 128, 0, st>>>((const double2*)tw64, (TwDF*)twdf, n);
     return (int)cudaGetLastError();
 }
-__global__ void k_v_to_df(const double* __restrict__ V, float2* __restrict__ out, long long N) {
+__global__ void k_v_to_df(const double* V, float2* __restrict__ out, long long N) {
     pdl_begin();
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (i < N) out[i] = df_split(V[i]);

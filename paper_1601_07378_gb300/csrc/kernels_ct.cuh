@@ -352,7 +352,7 @@ struct XRowsP {  // x rows at fixed y: the occupied planes
 // ------------------------------------------------------------------ K1
 template <int N, bool GM = false>
 __global__ void __launch_bounds__(kThreads, minb_k1(N)) k1_ct(DevTables t, const float2* __restrict__ tw3,
-                                                 const float2* __restrict__ coeffs, float2* __restrict__ cyl,
+                                                 const float2* coeffs, float2* __restrict__ cyl,
                                                  GammaArgs g) {
     pdl_begin();
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -379,7 +379,7 @@ __global__ void __launch_bounds__(kThreads, minb_k1(N)) k1_ct(DevTables t, const
 // formed from the caller's two real bands as they are read.
 template <int N, bool GM = false>
 __global__ void __launch_bounds__(kThreads, minb_k1(N)) k1q_ct(DevTables t, const float2* __restrict__ tw3,
-                                                  const float2* __restrict__ coeffs, float2* __restrict__ cyl,
+                                                  const float2* coeffs, float2* __restrict__ cyl,
                                                   GammaArgs g) {
     pdl_begin();
     using SC = Sched<N>;
@@ -483,7 +483,7 @@ __global__ void __launch_bounds__(kThreads, minb_k1(N)) k1q_ct(DevTables t, cons
 // instead of the dense table.
 template <int N, bool RUNS>
 __global__ void __launch_bounds__(kThreads, minb_k1(N)) k1d_ct(DevTables t, const float2* __restrict__ tw3,
-                                                  const float2* __restrict__ coeffs, float2* __restrict__ cyl) {
+                                                  const float2* coeffs, float2* __restrict__ cyl) {
     pdl_begin();
     using SC = Sched<N>;
     static_assert(SC::nst == 2, "quarter-band z-pass: two-stage lengths");
@@ -691,7 +691,7 @@ __global__ void __launch_bounds__(kThreads, minb_k2(N, S)) k2_ct(DevTables t, co
 // W warps per CTA (the tile is always 32 lines; more warps split its units).
 template <int N, int W>
 __global__ void __launch_bounds__(32 * W, minb_k3(N)) k3_ct(DevTables t, const float2* __restrict__ tw1,
-                                                 const float* __restrict__ Vr, float2* slab) {
+                                                 const float* Vr, float2* slab) {
     pdl_begin();
     using SC = Sched<N>;
     constexpr int nst = SC::nst;
@@ -809,7 +809,7 @@ constexpr int minb_k3q(int n) {
 // tiles without the per-lane division that maps a flat index to (y, z pair)).
 template <int N, int W, bool FLAT = true>
 __global__ void __launch_bounds__(32 * W, minb_k3q(N)) k3q_ct(DevTables t, const float2* __restrict__ tw1,
-                                                  const float* __restrict__ Vr, float2* slab) {
+                                                  const float* Vr, float2* slab) {
     pdl_begin();
     using SC = Sched<N>;
     static_assert(SC::nst == 2, "quarter-sphere x-pass: two-stage lengths");
@@ -977,8 +977,8 @@ __global__ void __launch_bounds__(32 * W, minb_k3q(N)) k3q_ct(DevTables t, const
 // ------------------------------------------------------------------ K4
 template <int N, bool GM = false>
 __global__ void __launch_bounds__(kThreads, minb_k4(N)) k4_ct(DevTables t, const float2* __restrict__ tw3,
-                                                 const float2* __restrict__ cyl, float2* out, float scale,
-                                                 const float* __restrict__ diag, const float2* cin, GammaArgs g) {
+                                                 const float2* cyl, float2* out, float scale,
+                                                 const float* diag, const float2* cin, GammaArgs g) {
     pdl_begin();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float2* buf = reinterpret_cast<float2*>(smem_raw);
@@ -1004,8 +1004,8 @@ __global__ void __launch_bounds__(kThreads, minb_k4(N)) k4_ct(DevTables t, const
 constexpr int minb_k4q(int n, bool gm) { return gm && n == 96 ? 7 : minb_k4(n); }
 template <int N, bool GM = false>
 __global__ void __launch_bounds__(kThreads, minb_k4q(N, GM)) k4q_ct(DevTables t, const float2* __restrict__ tw3,
-                                                  const float2* __restrict__ cyl, float2* out, float scale,
-                                                  const float* __restrict__ diag, const float2* cin, GammaArgs g) {
+                                                  const float2* cyl, float2* out, float scale,
+                                                  const float* diag, const float2* cin, GammaArgs g) {
     pdl_begin();
     using SC = Sched<N>;
     static_assert(SC::nst == 2, "quarter-band z-pass: two-stage lengths");
@@ -1061,8 +1061,8 @@ __global__ void __launch_bounds__(kThreads, minb_k4q(N, GM)) k4q_ct(DevTables t,
 constexpr int minb_k4d(int n) { return n == 96 ? 7 : minb_k4(n); }
 template <int N>
 __global__ void __launch_bounds__(kThreads, minb_k4d(N)) k4d_ct(DevTables t, const float2* __restrict__ tw3,
-                                                  const float2* __restrict__ cyl, float2* out, float scale,
-                                                  const float* __restrict__ diag, const float2* cin) {
+                                                  const float2* cyl, float2* out, float scale,
+                                                  const float* diag, const float2* cin) {
     pdl_begin();
     using SC = Sched<N>;
     static_assert(SC::nst == 2, "quarter-band z-pass: two-stage lengths");

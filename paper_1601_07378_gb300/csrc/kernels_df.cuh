@@ -110,7 +110,7 @@ template <class V> struct XRowsD {  // x rows at fixed y: the occupied planes
 // CTA (tile, band, half): lines [16 half, 16 half + 16) of the plan tile.
 template <class Pol, int N>
 __device__ __forceinline__ void k1w_body(const DevTables& t, const typename Pol::TW* __restrict__ tw3,
-                                         const double2* __restrict__ coeffs, typename Pol::V* __restrict__ cyl) {
+                                         const double2* coeffs, typename Pol::V* __restrict__ cyl) {
     using V = typename Pol::V;
     using TW = typename Pol::TW;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -169,13 +169,13 @@ template <class Pol, int N> constexpr bool df_floors() { return std::is_same<Pol
 #endif
 template <class Pol, int N>
 __global__ void __launch_bounds__(kThreads) k1_w(DevTables t, const typename Pol::TW* __restrict__ tw3,
-                                                const double2* __restrict__ coeffs, typename Pol::V* __restrict__ cyl) {
+                                                const double2* coeffs, typename Pol::V* __restrict__ cyl) {
     pdl_begin();
     k1w_body<Pol, N>(t, tw3, coeffs, cyl);
 }
 template <class Pol, int N, int MINB>
 __global__ void __launch_bounds__(kThreads, MINB) k1_wb(DevTables t, const typename Pol::TW* __restrict__ tw3,
-                                                       const double2* __restrict__ coeffs,
+                                                       const double2* coeffs,
                                                        typename Pol::V* __restrict__ cyl) {
     pdl_begin();
     k1w_body<Pol, N>(t, tw3, coeffs, cyl);
@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(kThreads, MINB) k1_wb(DevTables t, const typen
 // form's gather writes the caller's band in order.
 template <class Pol, int N>
 __device__ __forceinline__ void k1dw_body(const DevTables& t, const typename Pol::TW* __restrict__ tw3,
-                                          const double2* __restrict__ coeffs, typename Pol::V* __restrict__ cyl) {
+                                          const double2* coeffs, typename Pol::V* __restrict__ cyl) {
     using V = typename Pol::V;
     using TW = typename Pol::TW;
     using QR = QRows<N>;
@@ -250,13 +250,13 @@ __device__ __forceinline__ void k1dw_body(const DevTables& t, const typename Pol
 }
 template <class Pol, int N>
 __global__ void __launch_bounds__(kThreads) k1d_w(DevTables t, const typename Pol::TW* __restrict__ tw3,
-                                                 const double2* __restrict__ coeffs, typename Pol::V* __restrict__ cyl) {
+                                                 const double2* coeffs, typename Pol::V* __restrict__ cyl) {
     pdl_begin();
     k1dw_body<Pol, N>(t, tw3, coeffs, cyl);
 }
 template <class Pol, int N, int MINB>
 __global__ void __launch_bounds__(kThreads, MINB) k1d_wb(DevTables t, const typename Pol::TW* __restrict__ tw3,
-                                                        const double2* __restrict__ coeffs,
+                                                        const double2* coeffs,
                                                         typename Pol::V* __restrict__ cyl) {
     pdl_begin();
     k1dw_body<Pol, N>(t, tw3, coeffs, cyl);
@@ -344,7 +344,7 @@ __global__ void __launch_bounds__(kThreads, MINB) k2_wb(DevTables t, const typen
 // multiply and the first forward stage of the reversed schedule in registers.
 template <class Pol, int N>
 __global__ void __launch_bounds__(kThreads) k3_w(DevTables t, const typename Pol::TW* __restrict__ tw1,
-                                                const typename Pol::VR* __restrict__ Vr, typename Pol::V* slab) {
+                                                const typename Pol::VR* Vr, typename Pol::V* slab) {
     pdl_begin();
     using V = typename Pol::V;
     using TW = typename Pol::TW;
@@ -423,7 +423,7 @@ template <class Pol, int N> __host__ __device__ constexpr size_t k3q_w_smem() {
 }
 template <class Pol, int N>
 __global__ void __launch_bounds__(kThreads) k3q_w(DevTables t, const typename Pol::TW* __restrict__ tw1,
-                                                 const typename Pol::VR* __restrict__ Vr, typename Pol::V* slab) {
+                                                 const typename Pol::VR* Vr, typename Pol::V* slab) {
     pdl_begin();
     using V = typename Pol::V;
     using TW = typename Pol::TW;
@@ -533,8 +533,8 @@ __global__ void __launch_bounds__(kThreads) k3q_w(DevTables t, const typename Po
 // 0.268 -> 0.258 (72^3 x 256).
 template <class Pol, int N, bool Q>
 __device__ __forceinline__ void k4w_body(const DevTables& t, const typename Pol::TW* __restrict__ tw3,
-                                         const typename Pol::V* __restrict__ cyl, double2* out, double scale,
-                                         const double* __restrict__ diag, const double2* cin) {
+                                         const typename Pol::V* cyl, double2* out, double scale,
+                                         const double* diag, const double2* cin) {
     using V = typename Pol::V;
     using TW = typename Pol::TW;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -600,15 +600,15 @@ __device__ __forceinline__ void k4w_body(const DevTables& t, const typename Pol:
 
 template <class Pol, int N, bool Q>
 __global__ void __launch_bounds__(kThreads) k4_w(DevTables t, const typename Pol::TW* __restrict__ tw3,
-                                                const typename Pol::V* __restrict__ cyl, double2* out, double scale,
-                                                const double* __restrict__ diag, const double2* cin) {
+                                                const typename Pol::V* cyl, double2* out, double scale,
+                                                const double* diag, const double2* cin) {
     pdl_begin();
     k4w_body<Pol, N, Q>(t, tw3, cyl, out, scale, diag, cin);
 }
 template <class Pol, int N, bool Q, int MINB>
 __global__ void __launch_bounds__(kThreads, MINB) k4_wb(DevTables t, const typename Pol::TW* __restrict__ tw3,
-                                                       const typename Pol::V* __restrict__ cyl, double2* out,
-                                                       double scale, const double* __restrict__ diag,
+                                                       const typename Pol::V* cyl, double2* out,
+                                                       double scale, const double* diag,
                                                        const double2* cin) {
     pdl_begin();
     k4w_body<Pol, N, Q>(t, tw3, cyl, out, scale, diag, cin);

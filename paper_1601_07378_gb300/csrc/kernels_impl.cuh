@@ -118,7 +118,7 @@ __device__ __forceinline__ void rows_in(V* buf, const V* __restrict__ cb, const 
 // ------------------------------------------------------------------ K1
 template <typename T>
 __global__ void __launch_bounds__(kThreads) k1_scatter_zpass(DevTables t, AxisPlan az, const V2<T>* __restrict__ tw3,
-                                                            const V2<T>* __restrict__ coeffs, V2<T>* __restrict__ cyl) {
+                                                            const V2<T>* coeffs, V2<T>* __restrict__ cyl) {
     pdl_begin();
     using V = V2<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -213,7 +213,7 @@ template <typename T> struct TimesV {  // psi(x) * V(x, y, z) into shared memory
 
 template <typename T>
 __global__ void __launch_bounds__(kThreads) k3_xpass_v(DevTables t, AxisPlan ax, const V2<T>* __restrict__ tw1,
-                                                      const T* __restrict__ Vr, V2<T>* slab) {
+                                                      const T* Vr, V2<T>* slab) {
     pdl_begin();
     using V = V2<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -241,8 +241,8 @@ __global__ void __launch_bounds__(kThreads) k3_xpass_v(DevTables t, AxisPlan ax,
 // ------------------------------------------------------------------ K4
 template <typename T>
 __global__ void __launch_bounds__(kThreads) k4_zpass_gather(DevTables t, AxisPlan az, const V2<T>* __restrict__ tw3,
-                                                           const V2<T>* __restrict__ cyl, V2<T>* out, T scale,
-                                                           const T* __restrict__ diag, const V2<T>* cin) {
+                                                           const V2<T>* cyl, V2<T>* out, T scale,
+                                                           const T* diag, const V2<T>* cin) {
     pdl_begin();
     using V = V2<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];

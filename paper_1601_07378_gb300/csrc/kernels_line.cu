@@ -42,7 +42,7 @@ bool z_length(int n3) {
 
 // 32 x 32 tiles of (y, z) at one x through shared memory, so that both sides
 // are coalesced; 7 MB of traffic at 96^3 (about 3 us), once per call.
-__global__ void __launch_bounds__(256) k_vt(const float* __restrict__ V, float* __restrict__ VT, int n2, int n3) {
+__global__ void __launch_bounds__(256) k_vt(const float* V, float* __restrict__ VT, int n2, int n3) {
     pdl_begin();
     __shared__ float tile[32][33];
     const int z0 = blockIdx.x * 32, y0 = blockIdx.y * 32, x = blockIdx.z, n1 = gridDim.z;
@@ -90,7 +90,7 @@ int launch_dens(const Tables& t, const float2* D, long long nb, int bpg, const f
 }
 // Tiles of 32 (y, z) at one x: the partial sums read along y, the result
 // written along z.  Sum over the groups as in k_reduce_partials_f32.
-__global__ void __launch_bounds__(256) k_dens_reduce(const float* __restrict__ partial, int ng, int n2, int n3,
+__global__ void __launch_bounds__(256) k_dens_reduce(const float* partial, int ng, int n2, int n3,
                                                      double* __restrict__ acc, int first, float* __restrict__ out) {
     pdl_begin();
     __shared__ float ts[32][33], tc[32][33];

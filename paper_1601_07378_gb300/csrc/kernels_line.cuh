@@ -33,13 +33,17 @@ namespace line {
 __device__ __forceinline__ void bar_pair(int id) { asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory"); }
 
 // *p if lim >= k (k a constant), else 0; and the store: one compare and one
-// predicated access each (the compiler's own form branches around every load)
+// predicated access each (the compiler's own form branches around every load).
+// Volatile with a memory clobber: the dense rows are another launch's output
+// (pdl.cuh) and the step's own, so their loads keep their place among barriers
+// and stores.
 template <int k> __device__ __forceinline__ float2 ld_if_ge(const float2* p, int lim) {
     float2 v;
-    asm("{\n\t.reg .pred q;\n\tsetp.ge.s32 q, %3, %4;\n\tmov.f32 %0, 0f00000000;\n\tmov.f32 %1, 0f00000000;\n\t"
-        "@q ld.global.v2.f32 {%0, %1}, [%2];\n\t}"
-        : "=&f"(v.x), "=&f"(v.y)
-        : "l"(p), "r"(lim), "n"(k));
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ge.s32 q, %3, %4;\n\tmov.f32 %0, 0f00000000;\n\tmov.f32 %1, 0f00000000;\n\t"
+                 "@q ld.global.v2.f32 {%0, %1}, [%2];\n\t}"
+                 : "=&f"(v.x), "=&f"(v.y)
+                 : "l"(p), "r"(lim), "n"(k)
+                 : "memory");
     return v;
 }
 template <int k> __device__ __forceinline__ void st_if_ge(float2* p, float2 v, int lim) {
@@ -225,7 +229,7 @@ template <class C, int N2> __device__ __forceinline__ void yx_thin(bool fwd, con
 // Block (z, group of bpc bands), NBB bands at a time.
 template <int CLS, int N1, int N2>
 __global__ void __launch_bounds__(64 * YX<CLS, N1, N2>::PAIRS, YX<CLS, N1, N2>::MINB)
-    kl_yx(Tables t, const float2* __restrict__ tw2, const float* __restrict__ VT, int nb, int bpc, float2* D) {
+    kl_yx(Tables t, const float2* __restrict__ tw2, const float* VT, int nb, int bpc, float2* D) {
     pdl_begin();
     using C = YX<CLS, N1, N2>;
     constexpr int NBB = C::NBB;

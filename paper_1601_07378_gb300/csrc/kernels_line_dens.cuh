@@ -26,7 +26,7 @@ template <int CLS, int N1, int N2> struct YXD : YX<CLS, N1, N2> {
 
 template <int CLS, int N1, int N2>
 __global__ void __launch_bounds__(64 * YXD<CLS, N1, N2>::PAIRS, YXD<CLS, N1, N2>::MINB)
-    kl_dens(Tables t, const float2* __restrict__ D, int nb, int bpg, const float* __restrict__ occ, long long b_base,
+    kl_dens(Tables t, const float2* D, int nb, int bpg, const float* occ, long long b_base,
             int pair_mode, long long nreal, float* __restrict__ partial) {
     pdl_begin();
     using C = YXD<CLS, N1, N2>;

@@ -68,7 +68,7 @@ static_assert(kWarps % 2 == 0, "edge mapping: warps in pairs");
 // from the sticks' runs (caller lists in stick order), 2: Gamma-point pairs.
 template <int N, int MODE>
 __global__ void __launch_bounds__(kThreads, minb_k1(N)) kl_z_inv(Tables t, const float2* __restrict__ tw3,
-                                                            const float2* __restrict__ coeffs, long long nreal,
+                                                            const float2* coeffs, long long nreal,
                                                             float2* __restrict__ D) {
     pdl_begin();
     using SC = Sched<N>;
@@ -178,8 +178,8 @@ __global__ void __launch_bounds__(kThreads, minb_k1(N)) kl_z_inv(Tables t, const
 // pairs; times 1/N, plus diag times the band.  ED: see edge_slot.
 template <int N, bool GM, bool ED>
 __global__ void __launch_bounds__(kThreads, GM ? minb_k4q(N, true) : minb_k4d(N))
-    kl_z_fwd(Tables t, const float2* __restrict__ tw3, const float2* __restrict__ D, long long nreal, float2* out,
-             float scale, const float* __restrict__ diag, const float2* cin) {
+    kl_z_fwd(Tables t, const float2* __restrict__ tw3, const float2* D, long long nreal, float2* out,
+             float scale, const float* diag, const float2* cin) {
     pdl_begin();
     using SC = Sched<N>;
     static_assert(SC::nst == 2, "quarter-band z-pass: two-stage lengths");
