@@ -1511,11 +1511,13 @@ int vloc_density(vloc_plan p, const void* c, const void* occ, int64_t nb, void* 
 // the other way round where the kernels are the same (4 x 64 bands at 144^3 3.84
 // / 3.96) or short (60^3, 64^3, 72^3 x 256 0.827 / 0.857), and where the
 // instances do not fill the GPU (eight of 96^3 x 8 0.178 / 0.236; the count is
-// complex bands x z rows x y columns, the eight cubes with 4..32 bands lose from
-// 800 k on).
+// bands x z rows x y columns, the eight cubes with 4..32 bands lose from 800 k
+// on).  Gamma instances count their real bands, twice what their y/x pass runs:
+// 96^3 + 100^3 x 60 (30 pairs) 0.284 in turn / 0.295 on branches, 96^3, 100^3,
+// 108^3, 120^3 x 64 0.774 / 0.827, the eight cubes with 4..32 bands 0.645 / 0.682.
 static bool batch_apart(vloc_plan p, int64_t nb) {
-    const int64_t m = p->gamma ? (nb + 1) / 2 : nb;  // the bands of the y/x pass
-    return line_chunk(p, std::min<int64_t>(p->chunk, m)) && m * p->n3 * p->n2 >= 400000 && p->n1 + p->n2 >= 180;
+    return line_chunk(p, std::min<int64_t>(p->chunk, p->gamma ? (nb + 1) / 2 : nb)) &&
+           nb * p->n3 * p->n2 >= 400000 && p->n1 + p->n2 >= 180;
 }
 
 static int apply_batched(int ninst, const vloc_plan* plans, const void* const* c, const void* const* V,

@@ -164,10 +164,11 @@ done([create(8 << 30), create(2 << 30), create(256 << 20), [rt.cudaGetLastError(
 
 
 # Two large instances of different lengths: in turn on one branch if both run
-# the fused y/x pass on enough complex bands, else on two branches.
+# the fused y/x pass on enough bands, else on two branches.
 @pytest.mark.parametrize("bands,flags,chunk,branches", [
     (60, "VLOC_F32", 0, 1), (30, "VLOC_F32", 0, 2), (200, "VLOC_F32", 2, 2),    # chunk 2: five launches
-    (60, "VLOC_F32 | vloc.VLOC_GAMMA", 0, 2), (120, "VLOC_F32 | vloc.VLOC_GAMMA", 0, 1),    # 30 and 60 pairs
+    (60, "VLOC_F32 | vloc.VLOC_GAMMA", 0, 1), (30, "VLOC_F32 | vloc.VLOC_GAMMA", 0, 2),
+    (120, "VLOC_F32 | vloc.VLOC_GAMMA", 2, 2),
     (60, "VLOC_F64", 0, 2)])
 def test_batch_instances_in_turn_or_on_branches(run, bands, flags, chunk, branches):
     out = run(f"""
