@@ -33,6 +33,18 @@
  *    as void*, NULL = legacy default stream) and the call returns without
  *    synchronising, except where stated.  A plan must not be used by two
  *    streams at the same time.
+ *  - Rounding.  The same call gives the same bits.  A band's result does not
+ *    depend on the other bands' values (a VLOC_GAMMA band's on its pair's
+ *    alone), but which kernels run does depend on the number of bands: the
+ *    apply calls and the density of a VLOC_F32 plan go through three launches
+ *    (z-pass, fused y/x pass, z-pass) or five (z, y, x, y, z), by the plan and
+ *    by the bands of a launch, min(nbands, max_bands_per_chunk).  One band in
+ *    calls of different size, or under plans of different chunk, therefore
+ *    agrees to FP32 rounding (3e-7 in relative L2 between the two forms), not
+ *    bit for bit.  vloc_backward with grad_V, the half transforms,
+ *    vloc_apply_noalloc and plans with VLOC_X_TMA, VLOC_Z_WARP, VLOC_Z_BULK,
+ *    VLOC_GENERIC_KERNELS or a set schedule always take five launches; VLOC_F64
+ *    plans have only that form, and a band's result does not depend on the count.
  *  - Errors.  Every int-returning call returns VLOC_OK (0) or a negative
  *    VLOC_ERR_* code; no exception crosses this boundary.  On error nothing
  *    has been enqueued unless the code is VLOC_ERR_CUDA.
@@ -88,8 +100,9 @@ extern "C" {
                                        /* slab tiles move by TMA tensor copies,      */
                                        /* double-buffered on mbarriers (compiled x   */
                                        /* length, even n3; info.path bit 4).  Same   */
-                                       /* results bit for bit; measured slower than  */
-                                       /* the default x-pass at 96^3, kept opt-in.   */
+                                       /* results bit for bit as the five-launch     */
+                                       /* chain with the default x-pass; measured    */
+                                       /* slower at 96^3, kept opt-in.               */
                                        /* Its waits are bounded: see                 */
                                        /* vloc_device_status.                        */
 #define VLOC_Z_WARP             0x20000 /* FP32, n3 = 32, 64, 96 or 128, not Gamma: */
@@ -168,7 +181,8 @@ typedef struct vloc_info {
  *   max_bands_per_chunk : bands per workspace chunk (<= 0: automatic, a
  *                6 GiB workspace capped at 1/16 of the free device memory
  *                and at 2048 bands; large chunks keep every kernel many
- *                waves deep).
+ *                waves deep).  A given chunk whose workspace fits only
+ *                without the three-launch form makes a plan without it.
  *   stream     : stream used for the one-time table uploads (synchronised
  *                before return).
  * Errors: VLOC_ERR_ARG, VLOC_ERR_SIZE, VLOC_ERR_GLIST, VLOC_ERR_ALLOC,
@@ -233,7 +247,7 @@ int vloc_apply_adjoint(vloc_plan plan, const void* coeffs, const void* V, int64_
  *   path, FP64 in the FP64 path) whose partial sums are added in FP64 in a
  *   fixed order, so the result is deterministic.
  * Errors as vloc_apply; VLOC_ERR_STATE for a VLOC_GAMMA plan; VLOC_ERR_SIZE
- * when the dL/dV x-pass does not fit in shared memory (FP64, n1 > ~170).
+ * when the dL/dV x-pass does not fit in shared memory (FP64, n1 > 124).
  */
 int vloc_backward(vloc_plan plan, const void* coeffs, const void* grad_out, const void* V,
                   int64_t nbands, void* grad_coeffs, void* grad_V, void* stream);
@@ -281,8 +295,9 @@ int vloc_density(vloc_plan plan, const void* coeffs, const void* occ, int64_t nb
  * stream.  When every plan has VLOC_GRAPH the whole batch is captured once
  * (per pointer set) into one CUDA graph whose instances run as up to four
  * parallel branches (instances sharing a plan share a branch; large ones of
- * different lengths follow one another), and each call is one graph launch.  Arrays have ninst entries each; plans must
- * share a precision.  Errors as vloc_apply, per instance.
+ * different lengths follow one another), and each call is one graph launch.
+ * Arrays have ninst entries each; plans must share a precision.  Errors as
+ * vloc_apply, per instance.
  */
 int vloc_apply_batched(int ninst, const vloc_plan* plans, const void* const* coeffs,
                        const void* const* V, const int64_t* nbands, void* const* out,
@@ -342,9 +357,9 @@ int vloc_get_info(vloc_plan plan, vloc_info* info);
  * VLOC_HOST_ONLY plan (which made no CUDA call at all); together the two
  * never allocate device memory.  The caller passes inputs and outputs as
  * for vloc_apply (same layouts, alignment, alias and overlap rules).
- *   Kernels: the plan's own choice -- compile-time-length or runtime-radix
- *   kernels (VLOC_GENERIC_KERNELS, vloc_plan_set_schedule), and the
- *   double-float kernels for a VLOC_DOUBLE_FLOAT plan.
+ *   Kernels: the five-launch chain with the plan's own choice of
+ *   compile-time-length or runtime-radix kernels (VLOC_GENERIC_KERNELS,
+ *   vloc_plan_set_schedule), and the double-float kernels for a VLOC_DOUBLE_FLOAT plan.
  *   Not for VLOC_GAMMA plans: they return VLOC_ERR_STATE before any CUDA
  *   call is made.
  *   Limit: the tables, twiddles (for a double-float plan also V as hi + lo
