@@ -40,6 +40,46 @@ bool z_length(int n3) {
 #undef VLOC_CASE
 }
 
+// The y/x pass does the same work for a z whatever the sphere; the y- and
+// x-passes it replaces do less the fewer planes are occupied, and waste the rest
+// of their tiles of 32 z.  Their cost a z is about
+//     w (f + 1.1 - 0.2 q),  w = 32 ceil(n3 / 32) / n3,
+// in y-passes over all 2 (n1 / 4) + 1 planes, f of which are occupied and q = 1
+// where all are (the x-pass then knows them at compile time).  The table has the
+// cost, in twentieths, from which the y/x pass is the faster one: 0 where it
+// always was.  Gamma pairs cost their z-passes 6 % more.
+// Measured with both forms on every cell of these lengths within 1.35 of each
+// other, at f = 0.2 to 1, plain and Gamma (1848 pairs of times): always taking
+// the line path lost more than 1 % at 460 of them (up to 1.64: 128 x 96 x 96
+// with r = 6.5), the rule at 42 (up to 1.06); the density 310 (1.52) and 75 of
+// 1752 (1.13); among spheres that fill the smallest axis no more than 1.04.
+// Some, us for five launches / line path: 144^3 r = 9.5 568 / 763, r = 36 1068 /
+// 1000; 128^3 r = 18.5 617 / 648, r = 32 877 / 800, Gamma 894 / 923; 96^3 r = 8.5
+// 529 / 505; 72^3 r = 4.5 644 / 476; density 128^3 r = 18.5 404 / 439, 100^3 r =
+// 9.5 758 / 432.
+static const struct { unsigned char n1, n2, apply, density; } kPays[] = {
+    {24, 24, 41, 0}, {24, 32, 30, 0}, {32, 24, 38, 0}, {32, 32, 31, 0}, {48, 48, 33, 36},
+    {48, 60, 0, 30}, {48, 64, 0, 0}, {60, 48, 0, 28}, {60, 60, 0, 0}, {60, 64, 0, 0},
+    {60, 72, 0, 0}, {60, 80, 0, 0}, {64, 48, 31, 38}, {64, 60, 30, 35}, {64, 64, 32, 28},
+    {64, 72, 29, 39}, {64, 80, 29, 39}, {72, 60, 0, 28}, {72, 64, 0, 0}, {72, 72, 0, 39},
+    {72, 80, 0, 31}, {72, 96, 27, 28}, {80, 60, 28, 29}, {80, 64, 25, 0}, {80, 72, 31, 41},
+    {80, 80, 27, 33}, {80, 96, 28, 0}, {80, 100, 35, 40}, {96, 72, 35, 38}, {96, 80, 32, 34},
+    {96, 96, 28, 0}, {96, 100, 35, 37}, {96, 120, 32, 30}, {96, 128, 32, 28}, {100, 80, 47, 0},
+    {100, 96, 39, 0}, {100, 100, 37, 0}, {100, 120, 34, 0}, {100, 128, 37, 0}, {120, 96, 39, 0},
+    {120, 100, 37, 0}, {120, 120, 29, 0}, {120, 128, 29, 0}, {120, 144, 34, 0}, {128, 96, 40, 38},
+    {128, 100, 37, 59}, {128, 120, 32, 38}, {128, 128, 37, 38}, {128, 144, 37, 56}, {144, 120, 37, 0},
+    {144, 128, 40, 0}, {144, 144, 40, 29},
+};
+bool pays(int n1, int n2, int n3, int planes, bool gamma, bool density) {
+    const int all = 2 * (n1 / 4) + 1;
+    const double w = 32.0 * ((n3 + 31) / 32) / n3;
+    const double cost = w * ((double)planes / all + 1.1 - (planes == all ? 0.2 : 0.0));
+    for (const auto& k : kPays)
+        if (k.n1 == n1 && k.n2 == n2)
+            return 20.0 * cost >= (density ? (double)k.density : k.apply * (gamma ? 1.06 : 1.0));
+    return true;
+}
+
 // 32 x 32 tiles of (y, z) at one x through shared memory, so that both sides
 // are coalesced; 7 MB of traffic at 96^3 (about 3 us), once per call.
 __global__ void __launch_bounds__(256) k_vt(const float* V, float* __restrict__ VT, int n2, int n3) {

@@ -50,6 +50,9 @@ constexpr bool yx_thins(int n1, int n2) {
 // class index 0, 1, 2 (up to 48, 96, 144), or -1
 int yx_class(int n1, int n2);
 bool z_length(int n3);
+// Whether the form is the faster one for a cell of `planes` occupied x-planes
+// (lengths with compile-time five-launch kernels)
+bool pays(int n1, int n2, int n3, int planes, bool gamma, bool density);
 // elements between the k rows of the dense layout
 constexpr int class_pitch(int cls) { return cls == 0 ? 28 : cls == 1 ? 52 : 76; }
 

@@ -315,7 +315,7 @@ struct vloc_plan_s {
     size_t ws_bytes = 0;
     // line path (kernels_line.h): its tables; the dense bands share d_slab,
     // the transposed V the start of d_acc
-    bool line_on = false;
+    bool line_apply = false, line_density = false;  // calls that may take it
     vloc::line::Tables lt{};
     void* d_line = nullptr;
     size_t slab_bytes = 0;
@@ -786,7 +786,15 @@ static int create_plan(vloc_plan* out, int n1, int n2, int n3, const int32_t* g,
     // allocation-free entry runs the five-launch chain)
     LineHost lh;
     if (line_path && !dbl && p->fast && p->lay.zq && !(flags & (VLOC_X_TMA | VLOC_Z_WARP | VLOC_Z_BULK)) &&
-        std::getenv("VLOC_GAMMA_PACK") == nullptr)
+        std::getenv("VLOC_GAMMA_PACK") == nullptr) {
+        // where line::pays was measured; elsewhere the form is taken if it exists
+        // (a length without compile-time kernels: the five launches then take
+        // about twice as long; axes further apart: not cells of one spacing)
+        const bool known = has_ct(n1) && has_ct(n2) && has_ct(n3) && 20 * nmax <= 27 * std::min(n1, std::min(n2, n3));
+        p->line_apply = !known || line::pays(n1, n2, n3, NP, p->gamma, false);
+        p->line_density = !known || line::pays(n1, n2, n3, NP, p->gamma, true);
+    }
+    if (p->line_apply || p->line_density)
         lh = build_line(n1, n2, n3, stick_x, stick_row, stick_pw_ptr, pw_user, pw_z, gamma_neg, npw_user);
     // shared-memory budget of the largest kernel tile
     int dev = 0;
@@ -821,7 +829,8 @@ static int create_plan(vloc_plan* out, int n1, int n2, int n3, const int32_t* g,
         t.gamma = p->gamma; t.runs = lh.runs; t.trim = lh.trim;
         t.G = lh.G; t.n1 = n1; t.n2 = n2; t.n3 = n3; t.cls = lh.cls; t.npw = npw_user;
         t.row = (2 * (n2 / 4) + 1) * line::class_pitch(lh.cls);
-        p->line_on = true;
+    } else {
+        p->line_apply = p->line_density = false;
     }
     // the pair-forming z-passes exist for the FP32 compile-time kernels;
     // VLOC_GAMMA_PACK (a test aid) keeps the separate pack / unpack passes
@@ -847,7 +856,7 @@ static int create_plan(vloc_plan* out, int n1, int n2, int n3, const int32_t* g,
 
     // ---- workspace: cylinder [chunk][S][n3] + slab [chunk][NP][n2][n3], whose
     // place the line path's dense bands take
-    const size_t slab_elems = (size_t)NP * n2 * n3, dense_elems = p->line_on ? line::band_elems(p->lt) : 0;
+    const size_t slab_elems = (size_t)NP * n2 * n3, dense_elems = lh.cls >= 0 ? line::band_elems(p->lt) : 0;
     *grew = dense_elems > slab_elems;
     const size_t slab_band = std::max(slab_elems, dense_elems) * elem;
     const size_t per_band = (size_t)S * n3 * elem + slab_band;
@@ -949,7 +958,7 @@ int vloc_plan_set_schedule(vloc_plan p, int axis, int nst, const int32_t* radix)
     p->df = false;
     p->k3tma_on = false;
     p->gfused = false;
-    p->line_on = false;
+    p->line_apply = p->line_density = false;
     for (auto& g : p->graphs)
         if (g.exec) cudaGraphExecDestroy(g.exec);
     p->graphs.clear();
@@ -1025,16 +1034,15 @@ static int poison(vloc_plan p, cudaStream_t st) {
 
 extern "C" {
 
-// Whether a call whose first chunk holds cb bands goes through the line path,
-// by its dense z rows (n3 x bands): three blocks of the y/x pass an SM.
+// Whether a call whose first chunk holds cb bands has enough work for the line
+// path, by its dense z rows (n3 x bands): three blocks of the y/x pass an SM.
 // Measured against the five launches (us): 4 bands at 96^3 39.5 against 37.2,
 // 5 41.1 / 41.3, 7 43 / 49, 3 at 144^3 79 / 74, 4 85 / 87, 10 at 48^3 23.5 /
 // 28.2.  (Smaller grids would gain from 200 rows on, 5 bands at 48^3 22.8 /
 // 24.7; results then depend on the chunk size for more calls.)  An axis
 // without the five launches' compile-time kernels leaves them behind at any
 // count (6 bands at 36^3 37 against 22).
-static bool line_chunk(vloc_plan p, long long cb) {
-    if (!p->line_on) return false;
+static bool line_rows(vloc_plan p, long long cb) {
     return cb * p->n3 >= 456 || !(has_ct(p->n1) && has_ct(p->n2) && has_ct(p->n3));
 }
 static int line_vt(vloc_plan p, const void* V, cudaStream_t st) {
@@ -1081,7 +1089,7 @@ static int apply_impl(vloc_plan p, const void* c, const void* V, int64_t nb, voi
     }
     // the line path for all chunks of a call or none (a Gamma plan's packed
     // pairs, which come here, are not the caller's bands)
-    const bool line = !p->gamma && line_chunk(p, std::min<long long>(p->chunk, call_bands ? call_bands : nb));
+    const bool line = !p->gamma && p->line_apply && line_rows(p, std::min<long long>(p->chunk, call_bands ? call_bands : nb));
     if (line)
         if (int rc = line_vt(p, V, st)) return rc;
     for (int64_t b0 = 0; b0 < nb; b0 += p->chunk) {
@@ -1137,7 +1145,7 @@ static int gamma_apply(vloc_plan p, const void* c, const void* V, int64_t nb, vo
                        const void* diag) {
     const long long npairs = (nb + 1) / 2;
     // the line path for all chunks of a call or none
-    if (line_chunk(p, std::min<long long>(p->chunk, npairs))) {
+    if (p->line_apply && line_rows(p, std::min<long long>(p->chunk, npairs))) {
         if (int rc = line_vt(p, V, st)) return rc;
         const size_t ustride = (size_t)p->npw_user * p->elem;
         for (long long p0 = 0; p0 < npairs; p0 += p->chunk) {
@@ -1426,7 +1434,7 @@ int vloc_density(vloc_plan p, const void* c, const void* occ, int64_t nb, void* 
     // at 120^3, 1518 / 1526 at 128^3, 52.9 / 63.1 at 64^3 x 64.  Smaller groups
     // where the grid of 16-band groups leaves SMs idle (each group costs a
     // partial grid).
-    if (fused && p->n2 > 32 && line_chunk(p, std::min<long long>(p->chunk, p->gamma ? (nb + 1) / 2 : nb))) {
+    if (fused && p->line_density && p->n2 > 32 && line_rows(p, std::min<long long>(p->chunk, p->gamma ? (nb + 1) / 2 : nb))) {
         const long long pairs = p->gamma ? (nb + 1) / 2 : nb;  // complex bands
         float2* Dl = (float2*)p->d_slab;
         for (long long j0 = 0; j0 < pairs;) {
@@ -1516,7 +1524,7 @@ int vloc_density(vloc_plan p, const void* c, const void* occ, int64_t nb, void* 
 // 96^3 + 100^3 x 60 (30 pairs) 0.284 in turn / 0.295 on branches, 96^3, 100^3,
 // 108^3, 120^3 x 64 0.774 / 0.827, the eight cubes with 4..32 bands 0.645 / 0.682.
 static bool batch_apart(vloc_plan p, int64_t nb) {
-    return line_chunk(p, std::min<int64_t>(p->chunk, p->gamma ? (nb + 1) / 2 : nb)) &&
+    return p->line_apply && line_rows(p, std::min<int64_t>(p->chunk, p->gamma ? (nb + 1) / 2 : nb)) &&
            nb * p->n3 * p->n2 >= 400000 && p->n1 + p->n2 >= 180;
 }
 

@@ -226,3 +226,30 @@ done([codes, rt.fake_captures()])
 """)
     assert len(out[0]) > 5 and set(out[0][:-1]) == {-4} and out[0][-1] == 0
     assert out[1] == 0    # every capture that was begun was ended
+
+
+# Launches of an FP32 apply and a density of 64 bands (the line path: V's
+# transpose and three, and three; else five, and K1, K2, x-pass, reduction):
+# spheres well inside the quarter band of large grids, cells with one length
+# that suits the five launches, Gamma pairs, and what keeps the line path.
+@pytest.mark.parametrize("n,r,gamma,apply_line,density_line", [
+    ((144, 144, 144), 36, False, True, True), ((144, 144, 144), 12, False, False, True),
+    ((128, 128, 128), 32, False, True, True), ((128, 128, 128), 32, True, False, True),
+    ((128, 128, 128), 8, False, False, False), ((128, 96, 96), 24, False, False, False),
+    ((96, 96, 96), 24, False, True, True), ((96, 96, 96), 4, False, False, True),
+    ((100, 100, 100), 25, True, True, True), ((100, 100, 100), 6, False, False, True),
+    ((80, 80, 80), 10, False, True, True), ((64, 64, 64), 16, True, True, True), ((64, 64, 64), 4, False, False, False),
+    ((90, 96, 100), 3, False, True, None),        # a length without compile-time kernels
+    ((128, 128, 40), 10, False, True, True)])     # axes that are no cell's
+def test_line_path_where_it_pays(run, n, r, gamma, apply_line, density_line):
+    out = run(f"""
+h = plan({n!r}, {r}, vloc.VLOC_F32 | {"vloc.VLOC_GAMMA" if gamma else 0})
+l = [rt.fake_launches()]
+assert lib.vloc_apply(h, addr(0), addr(1), 128, addr(2), None) == 0
+l.append(rt.fake_launches())
+assert lib.vloc_density(h, addr(0), None, 128, addr(3), None) == 0
+l.append(rt.fake_launches())
+done([l[1] - l[0], l[2] - l[1]])
+""")
+    assert out[0] == (4 if apply_line else 5)
+    assert density_line is None or out[1] == (3 if density_line else 4)
