@@ -278,6 +278,7 @@ int launch_yx_n(const Tables& t, const float2* tw2, const float* VT, long long n
 // n1 = N1, every n2 of the class
 template <int CLS, int N1>
 int LaunchYX<CLS, N1>::run(const Tables& t, const float2* tw2, const float* VT, long long nb, float2* D, cudaStream_t st) {
+    static_assert(yx_partner(CLS, N1, yx_pair), "a length without kernels");
 #define VLOC_CASE(N) \
     case N:          \
         if constexpr (yx_pair(CLS, N1, N)) return launch_yx_n<CLS, N1, N>(t, tw2, VT, nb, D, st); \

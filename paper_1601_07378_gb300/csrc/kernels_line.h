@@ -24,7 +24,7 @@ namespace line {
 // per pair); the class fixes the pitch of the dense rows.
 #define VLOC_LINE_C48(X) X(24) X(30) X(32) X(36) X(40) X(48)
 #define VLOC_LINE_C96(X) X(48) X(50) X(54) X(60) X(64) X(72) X(80) X(90) X(96)
-#define VLOC_LINE_C144(X) X(72) X(80) X(90) X(96) X(100) X(108) X(120) X(128) X(144)
+#define VLOC_LINE_C144(X) X(80) X(90) X(96) X(100) X(108) X(120) X(128) X(144)
 // z lengths
 #define VLOC_LINE_Z_A(X) X(24) X(30) X(32) X(36) X(40) X(48)
 #define VLOC_LINE_Z_B(X) X(50) X(54) X(60) X(64) X(72) X(80)
@@ -47,6 +47,13 @@ constexpr bool yx_thins(int n1, int n2) {
     const int m = yx_bands(n1, n2), planes = 2 * (n1 / 4) + 1;
     return yx_rounds(m * (planes - 4)) < yx_rounds(m * planes);
 }
+// Whether n1 has a kernel with any n2 of the class
+#define VLOC_OR(N) || ok(cls, n1, N)
+template <class F> constexpr bool yx_partner(int cls, int n1, F ok) {
+    return (cls == 0 && (false VLOC_LINE_C48(VLOC_OR))) || (cls == 1 && (false VLOC_LINE_C96(VLOC_OR))) ||
+           (cls == 2 && (false VLOC_LINE_C144(VLOC_OR)));
+}
+#undef VLOC_OR
 // class index 0, 1, 2 (up to 48, 96, 144), or -1
 int yx_class(int n1, int n2);
 bool z_length(int n3);
@@ -104,9 +111,12 @@ template <int N> struct LaunchZ {
 };
 // the density of n1 with compile-time density kernels in the five-launch chain
 // (elsewhere the group sums are FP64)
-#define VLOC_LINE_D48(X) X(24) X(32) X(48)
+#define VLOC_LINE_D48(X) X(32) X(48)
 #define VLOC_LINE_D96(X) X(48) X(60) X(64) X(72) X(80) X(96)
-#define VLOC_LINE_D144(X) X(72) X(80) X(96) X(100) X(120) X(128) X(144)
+#define VLOC_LINE_D144(X) X(80) X(96) X(100) X(120) X(128) X(144)
+// and n2 whose lines fill both warp pairs of a block, which takes a band at a
+// time (32^3 x 300 bands 56 against 45 us)
+constexpr bool dens_pair(int cls, int n1, int n2) { return yx_pair(cls, n1, n2) && n2 > 32; }
 template <int CLS, int N1> struct LaunchDens {
     static int run(const Tables& t, const float2* D, long long nb, int bpg, const float* occ, long long b_base, int pair,
                    long long nreal, float* partial, cudaStream_t st);

@@ -1,9 +1,8 @@
-// kernels_line_da.cu -- density of the line path, n1 = 24, 32, 48, 48, 60, 64 (kernels_line.h).
+// kernels_line_da.cu -- density of the line path, n1 = 32, 48, 48, 60, 64 (kernels_line.h).
 #include "kernels_line_dens.cuh"
 
 namespace vloc {
 namespace line {
-template struct LaunchDens<0, 24>;
 template struct LaunchDens<0, 32>;
 template struct LaunchDens<0, 48>;
 template struct LaunchDens<1, 48>;

@@ -84,9 +84,10 @@ int launch_dens_n(const Tables& t, const float2* D, long long nb, int bpg, const
 template <int CLS, int N1>
 int LaunchDens<CLS, N1>::run(const Tables& t, const float2* D, long long nb, int bpg, const float* occ, long long b_base,
                              int pair, long long nreal, float* partial, cudaStream_t st) {
+    static_assert(yx_partner(CLS, N1, dens_pair), "a length without kernels");
 #define VLOC_CASE(N) \
     case N:          \
-        if constexpr (yx_pair(CLS, N1, N)) \
+        if constexpr (dens_pair(CLS, N1, N)) \
             return launch_dens_n<CLS, N1, N>(t, D, nb, bpg, occ, b_base, pair, nreal, partial, st); \
         else break;
     if constexpr (CLS == 0) switch (t.n2) { VLOC_LINE_C48(VLOC_CASE) default: break; }

@@ -1,4 +1,4 @@
-// kernels_line_yxk.cu -- y/x pass of the line path, size class 72 to 144, n1 = 128, 144 (kernels_line.h).
+// kernels_line_yxk.cu -- y/x pass of the line path, size class 80 to 144, n1 = 128, 144 (kernels_line.h).
 #include "kernels_line.cuh"
 
 namespace vloc {

@@ -1427,15 +1427,13 @@ int vloc_density(vloc_plan p, const void* c, const void* occ, int64_t nb, void* 
     const bool fused = pf32 && nb > 0;
     bool first = true;
     if (!fused && (rc = launch(p, KK_AUX, st, [&] { return launch_zero_f64(p->d_acc, p->N, st); }))) return rc;
-    // The line path's z-pass and y/x density pass, for all chunks or none.
-    // Its blocks take a band at a time, so n2 <= 32 leaves one of the two warp
-    // pairs idle (32^3 x 300 bands 56 against 45 us); above, the two ways
-    // measured 536 and 616 us at 96^3 x 300, 840 / 1197 at 100^3, 1210 / 1875
-    // at 120^3, 1518 / 1526 at 128^3, 52.9 / 63.1 at 64^3 x 64.  Smaller groups
-    // where the grid of 16-band groups leaves SMs idle (each group costs a
-    // partial grid).
-    if (fused && p->line_density && p->n2 > 32 && line_rows(p, std::min<long long>(p->chunk, p->gamma ? (nb + 1) / 2 : nb))) {
-        const long long pairs = p->gamma ? (nb + 1) / 2 : nb;  // complex bands
+    // The line path's z-pass and y/x density pass, for all chunks or none (536
+    // against 616 us at 96^3 x 300, 840 / 1197 at 100^3, 1210 / 1875 at 120^3,
+    // 52.9 / 63.1 at 64^3 x 64).  Smaller groups where the grid of 16-band
+    // groups leaves SMs idle (each group costs a partial grid).
+    const long long pairs = p->gamma ? (nb + 1) / 2 : nb;  // complex bands
+    if (fused && p->line_density && line::dens_pair(p->lt.cls, p->n1, p->n2) &&
+        line_rows(p, std::min<long long>(p->chunk, pairs))) {
         float2* Dl = (float2*)p->d_slab;
         for (long long j0 = 0; j0 < pairs;) {
             const long long cb = std::min(std::min<long long>(p->chunk, per_pass), pairs - j0);
