@@ -64,7 +64,7 @@ static const struct { unsigned char n1, n2, apply, density; } kPays[] = {
     {64, 72, 29, 39}, {64, 80, 29, 39}, {72, 60, 0, 28}, {72, 64, 0, 0}, {72, 72, 0, 39},
     {72, 80, 0, 31}, {72, 96, 27, 28}, {80, 60, 28, 29}, {80, 64, 25, 0}, {80, 72, 31, 41},
     {80, 80, 27, 33}, {80, 96, 28, 0}, {80, 100, 35, 40}, {96, 72, 35, 38}, {96, 80, 32, 34},
-    {96, 96, 28, 0}, {96, 100, 35, 37}, {96, 120, 32, 30}, {96, 128, 32, 28}, {100, 80, 47, 0},
+    {96, 96, 28, 26}, {96, 100, 35, 37}, {96, 120, 32, 30}, {96, 128, 32, 28}, {100, 80, 47, 0},
     {100, 96, 39, 0}, {100, 100, 37, 0}, {100, 120, 34, 0}, {100, 128, 37, 0}, {120, 96, 39, 0},
     {120, 100, 37, 0}, {120, 120, 29, 0}, {120, 128, 29, 0}, {120, 144, 34, 0}, {128, 96, 40, 38},
     {128, 100, 37, 59}, {128, 120, 32, 38}, {128, 128, 37, 38}, {128, 144, 37, 56}, {144, 120, 37, 0},
@@ -81,7 +81,7 @@ bool pays(int n1, int n2, int n3, int planes, bool gamma, bool density) {
 }
 
 // 32 x 32 tiles of (y, z) at one x through shared memory, so that both sides
-// are coalesced; 7 MB of traffic at 96^3 (about 3 us), once per call.
+// are coalesced; 7 MB of traffic at 96^3 (9 us with its launch), once per call.
 __global__ void __launch_bounds__(256) k_vt(const float* V, float* __restrict__ VT, int n2, int n3) {
     pdl_begin();
     __shared__ float tile[32][33];

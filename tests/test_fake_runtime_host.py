@@ -236,7 +236,7 @@ done([codes, rt.fake_captures()])
     ((144, 144, 144), 36, False, True, True), ((144, 144, 144), 12, False, False, True),
     ((128, 128, 128), 32, False, True, True), ((128, 128, 128), 32, True, False, True),
     ((128, 128, 128), 8, False, False, False), ((128, 96, 96), 24, False, False, False),
-    ((96, 96, 96), 24, False, True, True), ((96, 96, 96), 4, False, False, True),
+    ((96, 96, 96), 24, False, True, True), ((96, 96, 96), 4, False, False, False),
     ((100, 100, 100), 25, True, True, True), ((100, 100, 100), 6, False, False, True),
     ((80, 80, 80), 10, False, True, True), ((64, 64, 64), 16, True, True, True), ((64, 64, 64), 4, False, False, False),
     ((90, 96, 100), 3, False, True, None),        # a length without compile-time kernels
