@@ -13,14 +13,15 @@
 // non-coherent path or above the wait, and its inline loads of them are
 // volatile with a memory clobber.  Tables and twiddles, complete when the plan
 // is made, may be.  Neither costs anything: twelve workloads from 24^3 x 1 to
-// 96^3 x 1024 bands took the same time to 0.1 % with and without.  No kernel triggers its
-// successor early: blocks that wait take their place on the SMs unevenly while
-// the predecessor runs, which measured slower everywhere (below: GPU time per
-// apply in us without the attribute / early trigger / as it is).
-//   FP32  24^3 x 1  21.7 / 12.5 / 11.7    96^3 x 8   53.3 / 41.6 / 35.9
-//         48^3 x 20 32.9 / 20.6 / 16.4    96^3 x 512 1900 / 1726 / 1613
-//   (the first column: the five-launch chain, the others the line path)
-//   FP64  24^3 x 1  34.9 / 25.4 / 24.7    48^3 x 4   80 / 87 to 156 / 69
+// 96^3 x 1024 bands took the same time to 0.1 % with and without.
+// No kernel triggers its successor early: blocks that wait take their place on
+// the SMs unevenly while the predecessor runs, which measured slower everywhere.
+// us per apply, calls back to back, without the attribute / with it (with an
+// early trigger where the same chain was timed):
+//   FP32  five launches  24^3 x 1  22.6 / 12.4    48^3 x 8   26.0 / 15.3
+//         the line path  24^3 x 40 18.5 / 10.1    48^3 x 20  22.9 / 16.0 (20.6)
+//                        96^3 x 8  43.1 / 35.2 (41.6)   96^3 x 512 1618 / 1609 (1726)
+//   FP64  24^3 x 1  34.9 / 24.7 (25.4)    48^3 x 4   79.7 / 68.0 (87 to 156)
 #pragma once
 
 #include <cuda_runtime.h>

@@ -196,6 +196,10 @@ class VlocPlan:
     half of a G -> -G symmetric sphere, the bands are real in r-space
     (c(-G) = conj c(G) implied, c(0) taken real) and two of them share one
     complex transform.
+
+    FP32 results may differ in the last bits with the number of bands of a call
+    and with ``chunk``: blocks of enough bands run three fused launches, small
+    ones five (include/vloc.h, Rounding).
     """
 
     def __init__(self, grid, glist, dtype=None, *, partition: str = "greedy", chunk: int = 0,
