@@ -34,6 +34,7 @@ thread_local char g_last_cuda[256] = "";
 
 int cuda_fail(cudaError_t e, const char* what) {
     snprintf(g_last_cuda, sizeof(g_last_cuda), "%s: %s", what, cudaGetErrorString(e));
+    cudaGetLastError();  // reported here, not by a later launch's check
     return e == cudaErrorMemoryAllocation ? VLOC_ERR_ALLOC : VLOC_ERR_CUDA;
 }
 // f() for a C entry point: host memory that runs out is an error code there.
@@ -454,9 +455,7 @@ static int create_plan(vloc_plan* out, int n1, int n2, int n3, const int32_t* g,
     if (!p) return VLOC_ERR_ALLOC;
     auto dmalloc = [&](void** ptr, size_t bytes) -> cudaError_t {
         if (fault.alloc_at == alloc_no++) return cudaErrorMemoryAllocation;
-        const cudaError_t e = cudaMalloc(ptr, bytes);
-        if (e) cudaGetLastError();  // reported here, not by a later launch's check
-        return e;
+        return cudaMalloc(ptr, bytes);
     };
     p->poison = (flags & VLOC_POISON_WORKSPACE) != 0;
     p->n1 = n1; p->n2 = n2; p->n3 = n3; p->dbl = dbl; p->flags = flags; p->npw = npw; p->N = N;
@@ -994,27 +993,33 @@ static int check_io(vloc_plan p, const void* c, const void* V, int64_t nb, const
 
 }  // extern "C"
 
+// Two timing events for one more launch of `kind`.
+static int prof_begin(vloc_plan p, int kind) {
+    const size_t i0 = p->prof_recs.size() * 2;
+    while (p->prof_pool.size() < i0 + 2) {
+        if (p->prof_pool.size() == p->prof_pool.capacity()) p->prof_pool.reserve(2 * p->prof_pool.size() + 64);
+        cudaEvent_t e;
+        cudaError_t err = cudaEventCreate(&e);
+        if (err) return cuda_fail(err, "profiling event");
+        p->prof_pool.push_back(e);
+    }
+    p->prof_recs.push_back({kind, i0});
+    return VLOC_OK;
+}
 // Launch one kernel of the chain, bracketed by timing events when profiling.
 template <class F>
 static int launch(vloc_plan p, int kind, cudaStream_t st, F&& f) {
-    size_t i0 = 0;
     if (p->prof_on) {
-        i0 = p->prof_recs.size() * 2;
-        while (p->prof_pool.size() < i0 + 2) {
-            cudaEvent_t e;
-            cudaError_t err = cudaEventCreate(&e);
-            if (err) return cuda_fail(err, "profiling event");
-            p->prof_pool.push_back(e);
-        }
-        cudaEventRecord(p->prof_pool[i0], st);
+        if (int rc = guarded([&] { return prof_begin(p, kind); })) return rc;
+        cudaEventRecord(p->prof_pool[p->prof_recs.back().second], st);
     }
     const int rc = f();
-    if (rc) return cuda_fail((cudaError_t)rc, "kernel launch");
-    ++p->launches;
-    if (p->prof_on) {
-        cudaEventRecord(p->prof_pool[i0 + 1], st);
-        p->prof_recs.push_back({kind, i0});
+    if (rc) {
+        if (p->prof_on) p->prof_recs.pop_back();
+        return cuda_fail((cudaError_t)rc, "kernel launch");
     }
+    ++p->launches;
+    if (p->prof_on) cudaEventRecord(p->prof_pool[p->prof_recs.back().second + 1], st);
     return VLOC_OK;
 }
 
@@ -1735,11 +1740,11 @@ static int apply_host_impl(vloc_plan p, const void* ch, const void* Vh, int64_t 
 }
 
 int vloc_apply_host(vloc_plan p, const void* ch, const void* Vh, int64_t nb, void* oh, void* stream) {
-    return apply_host_impl(p, ch, Vh, nb, oh, stream, true);
+    return guarded([&] { return apply_host_impl(p, ch, Vh, nb, oh, stream, true); });
 }
 
 int vloc_apply_host_async(vloc_plan p, const void* ch, const void* Vh, int64_t nb, void* oh, void* stream) {
-    return apply_host_impl(p, ch, Vh, nb, oh, stream, false);
+    return guarded([&] { return apply_host_impl(p, ch, Vh, nb, oh, stream, false); });
 }
 
 int vloc_device_status(vloc_plan p) {

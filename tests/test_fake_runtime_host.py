@@ -253,3 +253,32 @@ done([l[1] - l[0], l[2] - l[1]])
 """)
     assert out[0] == (4 if apply_line else 5)
     assert density_line is None or out[1] == (3 if density_line else 4)
+
+
+@pytest.mark.parametrize("call", ["lib.vloc_apply(h, addr(0), addr(1), 20, addr(2), None)",    # profiled
+                                  "lib.vloc_apply_host(h, addr(0), addr(1), 4000, addr(2), None)"])
+def test_memory_that_runs_out_in_a_call_is_an_error_code(run, call):
+    """Host allocations of the profiling records and of the staging schedule,
+    and the device allocation of the staging buffers: VLOC_ERR_ALLOC, the call
+    works afterwards, and no CUDA error is left for a later launch check."""
+    out = run(f"""
+h = plan((48, 48, 48), 12, vloc.VLOC_F32)
+assert lib.vloc_profile(h, 1) == 0
+call = lambda: {call}
+codes, k = [], 0
+if "host" in {call!r}:
+    rt.fake_set_free(1 << 20)
+    codes.append(call())
+    rt.fake_set_free(64 << 30)
+while not codes or codes[-1]:
+    rt.fake_new_at(k)
+    codes.append(call())
+    rt.fake_new_at(-1)
+    k += 1
+n = ctypes.c_int64()
+stats = (vloc.VlocKernelStat * 12)()
+assert lib.vloc_get_profile(h, stats) == 0
+done([codes, call(), rt.cudaGetLastError(), sum(x.launches for x in stats)])
+""")
+    assert len(out[0]) >= 3 and set(out[0][:-1]) == {-4} and out[0][-1] == 0
+    assert out[1:3] == [0, 0] and out[3] >= 4
